@@ -23,8 +23,8 @@
 // theta = (lengthscale, sigma2, nugget); theta_bar is accumulated in FP64.
 #include <algorithm>
 
+#include "pointpair.cuh"
 #include "pointwide.cuh"
-#include "sweepsync.cuh"
 
 namespace ggp {
 namespace {
@@ -459,235 +459,177 @@ __global__ void __launch_bounds__(128) factor_backward_rescue_kernel(
   block_add3(tl, ts, tn, thetabar);
 }
 
-// The per-row factor backward of one-thread-per-point rows, after
-// point_factor_thread left the row's factor in p and its coordinates in the
-// stage: g = K_cc^-1 (alpha v_c), then Kbar against dkappa/dtheta over the
-// pairs.  Once g is solved, L is dead and the coordinates are reloaded for
-// the kernel derivatives; the pair (a, c), c < a, takes Kbar_ac + Kbar_ca
-// against the symmetric dkappa_ac.  Each row's sum (FP32, at most k + 1
-// terms) goes straight into the thread's FP64 totals.
+// The per-row backward for k <= 16: two lanes per point, the factor recomputed
+// by pair_factor (bit-identical b and sigma to the forward kernel).
 template <int K, int KT>
-__device__ __forceinline__ void thread_row_backward(PointRegs<K>& p, const ThreadStage<K>& st,
-                                                    const int32_t* row_ptr, int k,
-                                                    const KernF& kf, float4 xq,
-                                                    const float* __restrict__ v, float alpha,
-                                                    float sbar, double& tl, double& ts,
-                                                    double& tn) {
-  const float inv_s2 = 1.0f / kf.s2;
-  const int4* row = reinterpret_cast<const int4*>(row_ptr);
-  float g[K];
-  int32_t ca[K];
-#pragma unroll
-  for (int q = 0; q < K / 4; q++) {
-    const int4 c = __ldg(row + q);
-    ca[4 * q] = c.x;
-    ca[4 * q + 1] = c.y;
-    ca[4 * q + 2] = c.z;
-    ca[4 * q + 3] = c.w;
-  }
-#pragma unroll
-  for (int a = 0; a < K; a++) g[a] = a < k ? alpha * v[ca[a]] : 0.0f;
-  thread_chol_solve<K>(p, k, g);
-  // b and g into the stage (the kernel values there are consumed), then a
-  // rolled loop over the pairs: row sums in FP32 (at most k + 1 terms),
-  // added to the FP64 totals
-  float* sb = st.E;
-  float* sg = st.E + K * kThreadBlock;
-#pragma unroll
-  for (int a = 0; a < K; a++) {
-    sb[a * kThreadBlock] = p.y[a];
-    sg[a * kThreadBlock] = g[a];
-  }
-  ts += sbar;  // Kbar_ii = sbar
-  tn += sbar;
-#pragma unroll 1
-  for (int a = 0; a < k; a++) {
-    const float ga = sg[a * kThreadBlock], ba = sb[a * kThreadBlock];
-    const float4 xa = st.X[a * kThreadBlock];
-    {
-      const float kaa = -ga * ba + sbar * ba * ba;
-      float pl = 0.0f, ps = kaa;
-      int c = 0;
-      // four pairs per iteration, evaluated together and added in order
-#pragma unroll 1
-      for (; c + 4 <= a; c += 4) {
-        float gc[4], bc[4];
-        float4 xc[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-          gc[u] = sg[(c + u) * kThreadBlock];
-          bc[u] = sb[(c + u) * kThreadBlock];
-          xc[u] = st.X[(c + u) * kThreadBlock];
-        }
-        float kb[4];
-        KD kd[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-          kb[u] = (-ga * bc[u] + sbar * ba * bc[u]) + (-gc[u] * ba + sbar * bc[u] * ba);
-          kd[u] = kappa_dkappa_d2<KT>(kf, sqdist(xa, xc[u]));
-        }
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-          ps += kb[u] * kd[u].k * inv_s2;
-          pl += kb[u] * kd[u].dl;
-        }
-      }
-#pragma unroll 1
-      for (; c < a; c++) {
-        const float gc = sg[c * kThreadBlock], bc = sb[c * kThreadBlock];
-        const float kb = (-ga * bc + sbar * ba * bc) + (-gc * ba + sbar * bc * ba);
-        const KD kd = kappa_dkappa_d2<KT>(kf, sqdist(xa, st.X[c * kThreadBlock]));
-        ps += kb * kd.k * inv_s2;
-        pl += kb * kd.dl;
-      }
-      const float kci = ga - 2.0f * sbar * ba;
-      const KD kq = kappa_dkappa_d2<KT>(kf, sqdist(xa, xq));
-      ps += kci * kq.k * inv_s2;
-      pl += kci * kq.dl;
-      tl += pl;
-      ts += ps;
-      tn += kaa;
-    }
-  }
-}
-
-// The same per-row backward with one thread per point and the factor in
-// registers (k <= 16, K = padded row length), recomputed by
-// point_factor_thread: bit-identical b and sigma to the forward kernel.
-template <int K, int KT>
-__global__ void __launch_bounds__(128) factor_backward_thread_kernel(
+__global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) factor_backward_pair_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int64_t n0,
     KernF kf, int mode, const float* __restrict__ coef, float beta, const float* __restrict__ v,
     const float* __restrict__ xi, float* __restrict__ xibar_out, double* __restrict__ thetabar,
     int64_t* __restrict__ rescue_rows, unsigned long long* __restrict__ rescue_count,
     unsigned long long rescue_cap) {
-  extern __shared__ __align__(16) unsigned char tstage[];
-  const ThreadStage<K> st(tstage);
-  double tl = 0.0, ts = 0.0, tn = 0.0;
+  using PL = PairLayout<K>;
+  extern __shared__ __align__(16) float psm[];
+  const int lane = threadIdx.x & 31, r = lane & 1, first = (threadIdx.x >> 5) * 16;
+  float* S = psm + (threadIdx.x >> 1) * PL::kStride;
+  const uint64_t pol_v = l2_evict_last();
+  double tl = 0.0, ts = 0.0, tn = 0.0;   // scaled sums of the FP32 rows
+  double wl = 0.0, ws = 0.0, wn = 0.0;   // rows recomputed here in FP64
   const int64_t npts = N - n0;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < npts;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = n0 + t;
-    const int32_t* row_ptr = nbr + t * K;
+  const int64_t stride = (int64_t)gridDim.x * PL::kPoints;
+  PairLoad<K> ld;
+  for (int64_t b0 = (int64_t)blockIdx.x * PL::kPoints; b0 < npts; b0 += stride) {
+    __syncthreads();  // the warps of a block share the instruction stream
+    const int64_t t = b0 + first + (lane >> 1);
+    const bool valid = t < npts;
+    const int64_t tt = valid ? t : npts - 1, i = n0 + tt;
+    const int32_t* row_ptr = nbr + tt * K;
     const float4 xq = __ldg(xs + i);
-    PointRegs<K> p;
-    stage_coords<K>(st, xs, row_ptr, k);
-    point_factor_thread<K, KT>(p, k, kf, st, xq);
-    if (needs_rescue(p, k, kf)) {
+    ld.indices(r, row_ptr);
+    ld.coords(r, xs);
+    ld.stage(S, r);
+    PairFactor<K> f;
+    pair_factor<K, KT>(f, S, r, k, kf, xq);
+    const bool rescue = valid && pair_needs_rescue(f, kf);
+    const float ci = coef[i], xii = xi[i];
+    const float alpha = mode == 0 ? -ci / f.sigma : ci;
+    const float sigbar = alpha * xii + beta / f.sigma;
+    float vv[K / 2];
+    pair_gather<K, false>(vv, r, row_ptr, v, pol_v);
+    pair_row_backward<K, KT>(f, S, r, k, kf, xq, vv, alpha, sigbar / (2.0f * f.sigma),
+                             valid && !rescue, tl, ts, tn);
+    if (valid && !rescue && r == 0 && mode == 1) xibar_out[i] = f.sigma * ci;
+    if (rescue && r == 0) {
       // listed for factor_backward_rescue_kernel; recomputed here when the list is full
       const unsigned long long slot = atomicAdd(rescue_count, 1ull);
       if (slot < rescue_cap) {
         rescue_rows[slot] = i;
-        continue;
+      } else {
+        Row64<K> R;
+        row_factor64<K, KT>(R, xs, row_ptr, k, xq, kf);
+        const float sg = (float)R.sigma;
+        const double al = mode == 0 ? -(double)ci / sg : (double)ci;
+        const double sb = al * (double)xii + (double)beta / sg;
+        row_backward64<K, KT>(R, xs, row_ptr, k, xq, kf, v, al, sb, sg, wl, ws, wn);
+        if (mode == 1) xibar_out[i] = sg * ci;
       }
-      Row64<K> R;
-      row_factor64<K, KT>(R, xs, row_ptr, k, xq, kf);
-      const float sg = (float)R.sigma;
-      const float ci = coef[i];
-      const double alpha = mode == 0 ? -(double)ci / sg : (double)ci;
-      const double sigbar = alpha * (double)xi[i] + (double)beta / sg;
-      row_backward64<K, KT>(R, xs, row_ptr, k, xq, kf, v, alpha, sigbar, sg, tl, ts, tn);
-      if (mode == 1) xibar_out[i] = sg * ci;
-      continue;
     }
-    const float sigma = p.sigma;
-    const float ci = coef[i];
-    const float alpha = mode == 0 ? -ci / sigma : ci;
-    const float sigbar = alpha * xi[i] + beta / sigma;
-    thread_row_backward<K, KT>(p, st, row_ptr, k, kf, xq, v, alpha, sigbar / (2.0f * sigma), tl,
-                               ts, tn);
-    if (mode == 1) xibar_out[i] = sigma * ci;
+    __syncwarp();
   }
-  block_add3(tl, ts, tn, thetabar);
+  block_add3(wl + tl * theta_scale<KT>(kf), ws + ts, wn + tn, thetabar);
 }
 
 // NLL value and gradient in one pass, the factors recomputed and never stored
-// (k <= 16, one thread per point).  Each row's b and sigma come from
-// point_factor_thread with the factor kernel's FP64 rescue (warp_rescue), so
-// they are bit-identical to a stored factor's; xi_i = (v_i - b . v_c) /
-// sigma_i follows the stored sweeps' order.  The row then adds its share of
-// what graphgp_nll + graphgp_nll_backward compute: xi_i^2 and log sigma_i
-// to the value; w_i = nllbar xi_i / sigma_i at i and -w_i b_ia at each
-// neighbour (vbar, atomic adds; vbar's sparse entries start at 0); and the
-// row's factor backward with alpha = -w_i and sigbar = alpha xi_i +
-// nllbar / sigma_i (the logdet cotangent nllbar / 2, doubled).  Rows sent to
-// FP64 leave xi_i and nllbar xi_i in xi_out / xibar_out and are listed for
+// (k <= 16, two lanes per point).  Each row's b and sigma come from pair_factor
+// with the factor kernel's FP64 rescue, so they are bit-identical to a stored
+// factor's; xi_i = (v_i - b . v_c) / sigma_i follows the stored sweeps' order.
+// The row then adds its share of what graphgp_nll + graphgp_nll_backward
+// compute: xi_i^2 and log sigma_i to the value; w_i = nllbar xi_i / sigma_i at
+// i and -w_i b_ia at each neighbour (vbar, atomic adds; vbar's sparse entries
+// start at 0); and the row's factor backward with alpha = -w_i and sigbar =
+// alpha xi_i + nllbar / sigma_i (the logdet cotangent nllbar / 2, doubled).
+// Rows sent to FP64 follow the others of their warp, one at a time: they leave
+// xi_i and nllbar xi_i in xi_out / xibar_out and are listed for
 // factor_backward_rescue_kernel (recomputed here when the list is full).
-// Iterations are uniform across the warp (warp_rescue is a collective).
 template <int K, int KT>
-__global__ void __launch_bounds__(128) nll_grad_fused_kernel(
+__global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) nll_grad_fused_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int64_t n0,
     KernF kf, float nllbar, const float* __restrict__ v, float* vbar, float* __restrict__ xi_out,
     float* __restrict__ xibar_out, double* __restrict__ thetabar, double* __restrict__ acc,
     unsigned long long* __restrict__ not_pd, int64_t* __restrict__ rescue_rows,
     unsigned long long* __restrict__ rescue_count, unsigned long long rescue_cap) {
-  extern __shared__ __align__(16) unsigned char tstage[];
-  const ThreadStage<K> st(tstage);
-  double* W = fused_rescue_ws<K>(tstage);
+  using PL = PairLayout<K>;
+  extern __shared__ __align__(16) float psm[];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, r = lane & 1, first = (threadIdx.x >> 5) * 16;
+  float* S = psm + (threadIdx.x >> 1) * PL::kStride;
   const uint64_t pol_v = l2_evict_last();
   LogAcc lacc;
-  double sq = 0.0, tl = 0.0, ts = 0.0, tn = 0.0;
+  double sq = 0.0, tl = 0.0, ts = 0.0, tn = 0.0, wl = 0.0, ws = 0.0, wn = 0.0;
   unsigned long long clamped = 0;
   const int64_t npts = N - n0;
-  const int64_t total = (int64_t)gridDim.x * blockDim.x;
-  const int64_t iters = (npts + total - 1) / total;  // the same on every lane
-  for (int64_t it = 0; it < iters; it++) {
-    const int64_t t = it * total + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * PL::kPoints;
+  PairLoad<K> ld;
+  for (int64_t b0 = (int64_t)blockIdx.x * PL::kPoints; b0 < npts; b0 += stride) {
+    __syncthreads();  // the warps of a block share the instruction stream
+    const int64_t t = b0 + first + (lane >> 1);
     const bool valid = t < npts;
-    const int64_t i = n0 + (valid ? t : 0);
-    const int32_t* row_ptr = nbr + (valid ? t : 0) * K;
+    const int64_t tt = valid ? t : npts - 1, i = n0 + tt;
+    const int32_t* row_ptr = nbr + tt * K;
     const float4 xq = __ldg(xs + i);
-    PointRegs<K> p;
-    if (valid) {
-      stage_coords<K>(st, xs, row_ptr, k);
-      point_factor_thread<K, KT>(p, k, kf, st, xq);
-    }
-    const bool rescue = valid && needs_rescue(p, k, kf);
-    warp_rescue<K, KT>(p, rescue, xs, row_ptr, k, xq, kf, W);
-    if (!valid) continue;
-    const float sigma = p.sigma;
-    const float xv = (ld_keep_f(v + i, pol_v) - dot_stored_order<K, false>(p.y, row_ptr, v, pol_v)) / sigma;
-    sq += (double)xv * (double)xv;
-    lacc.mul(sigma);
-    clamped += p.clamped ? 1 : 0;
+    ld.indices(r, row_ptr);
+    ld.coords(r, xs);
+    ld.stage(S, r);
+    PairFactor<K> f;
+    pair_factor<K, KT>(f, S, r, k, kf, xq);
+    const bool rescue = valid && pair_needs_rescue(f, kf), act = valid && !rescue;
+    float vv[K / 2];
+    pair_gather<K, false>(vv, r, row_ptr, v, pol_v);
+    const float sigma = f.sigma;
+    const float xv = (ld_keep_f(v + i, pol_v) - pair_dot<K>(f.b, vv, r)) / sigma;
     const float xb = nllbar * xv;
     const float w = xb / sigma;
-    atomicAdd(vbar + i, w);
-#pragma unroll
-    for (int q = 0; q < K / 4; q++) {
-      const int4 c = __ldg(reinterpret_cast<const int4*>(row_ptr) + q);
-      if (p.y[4 * q] != 0.0f) atomicAdd(vbar + c.x, p.y[4 * q] * -w);
-      if (p.y[4 * q + 1] != 0.0f) atomicAdd(vbar + c.y, p.y[4 * q + 1] * -w);
-      if (p.y[4 * q + 2] != 0.0f) atomicAdd(vbar + c.z, p.y[4 * q + 2] * -w);
-      if (p.y[4 * q + 3] != 0.0f) atomicAdd(vbar + c.w, p.y[4 * q + 3] * -w);
-    }
-    if (rescue) {
-      xi_out[i] = xv;
-      xibar_out[i] = xb;
-      const unsigned long long slot = atomicAdd(rescue_count, 1ull);
-      if (slot < rescue_cap) {
-        rescue_rows[slot] = i;
-        continue;
+    if (act) {
+      if (r == 0) {
+        sq += (double)xv * (double)xv;
+        lacc.mul(sigma);
+        clamped += f.clamped ? 1 : 0;
+        atomicAdd(vbar + i, w);
       }
-      Row64<K> R;
-      row_factor64<K, KT>(R, xs, row_ptr, k, xq, kf);
-      const float sg = (float)R.sigma;
-      const double alpha = -(double)xb / sg;
-      const double sigbar = alpha * (double)xv + (double)nllbar / sg;
-      row_backward64<K, KT>(R, xs, row_ptr, k, xq, kf, v, alpha, sigbar, sg, tl, ts, tn);
-      continue;
+#pragma unroll
+      for (int s = 0; s < K / 2; s++) {
+        const int2 c = __ldg(reinterpret_cast<const int2*>(row_ptr) + s);
+        const float bs = pair_own<K>(f.b, r, s);
+        if (bs != 0.0f) atomicAdd(vbar + (r ? c.y : c.x), bs * -w);
+      }
     }
     const float alpha = -xb / sigma;
     const float sigbar = alpha * xv + nllbar / sigma;
-    thread_row_backward<K, KT>(p, st, row_ptr, k, kf, xq, v, alpha, sigbar / (2.0f * sigma), tl,
-                               ts, tn);
+    pair_row_backward<K, KT>(f, S, r, k, kf, xq, vv, alpha, sigbar / (2.0f * sigma), act, tl, ts,
+                             tn);
+    unsigned m = __ballot_sync(full, rescue && r == 0);
+    while (m) {
+      const int src = __ffs(m) - 1;
+      m &= m - 1;
+      __syncwarp();
+      const int64_t u = b0 + first + (src >> 1), iu = n0 + u;
+      const int32_t* row = nbr + u * K;
+      const float4 xu = __ldg(xs + iu);
+      const WarpRow64 wr = warp_row_factor64<K, KT>(
+          xs, row, k, xu, kf, reinterpret_cast<double*>(psm + first * PL::kStride));
+      const float b = lane < k ? (float)wr.b : 0.0f, sg = (float)wr.sigma;
+      const float dot = warp_dot_stored_order<K, false>(b, row, v, pol_v);
+      const float xu0 = __shfl_sync(full, (ld_keep_f(v + iu, pol_v) - dot) / sg, 0);
+      const float xbu = nllbar * xu0, wu = xbu / sg;
+      if (lane < k && b != 0.0f) atomicAdd(vbar + row[lane], b * -wu);
+      if (lane == src) {
+        sq += (double)xu0 * (double)xu0;
+        lacc.mul(sg);
+        clamped += wr.clamped ? 1 : 0;
+        atomicAdd(vbar + iu, wu);
+        xi_out[iu] = xu0;
+        xibar_out[iu] = xbu;
+        const unsigned long long slot = atomicAdd(rescue_count, 1ull);
+        if (slot < rescue_cap) {
+          rescue_rows[slot] = iu;
+        } else {
+          Row64<K> R;
+          row_factor64<K, KT>(R, xs, row, k, xu, kf);
+          const float s64 = (float)R.sigma;
+          const double al = -(double)xbu / s64;
+          const double sb = al * (double)xu0 + (double)nllbar / s64;
+          row_backward64<K, KT>(R, xs, row, k, xu, kf, v, al, sb, s64, wl, ws, wn);
+        }
+      }
+    }
+    __syncwarp();
   }
-  block_add3(tl, ts, tn, thetabar);
+  block_add3(wl + tl * theta_scale<KT>(kf), ws + ts, wn + tn, thetabar);
   block_add_double(sq, acc);
   block_add_double(lacc.log_value(), acc + 1);
   unsigned long long c = clamped;
-  for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(not_pd, c);
+  for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(full, c, o);
+  if (lane == 0 && c) atomicAdd(not_pd, c);
 }
 
 // The FP64 conditional of a warp's row out of line: the rescue is rare, and
@@ -843,13 +785,13 @@ int launch_factor_backward(graphgp_graph_t g, graphgp_factor_t f, int mode, cons
 constexpr int64_t kBackwardRescueMax = 1 << 20;  // rows listed for the FP64 backward
 
 template <int K>
-int launch_factor_backward_thread(graphgp_graph_t g, graphgp_factor_t f, int mode,
+int launch_factor_backward_pair(graphgp_graph_t g, graphgp_factor_t f, int mode,
                                   const float* coef, float beta, const float* v, const float* xi,
                                   float* xibar, double* thetabar, const int32_t* nbr,
                                   int64_t N, int64_t n0v, cudaStream_t s) {
   const int64_t npts = N - n0v;
   if (npts <= 0) return GRAPHGP_OK;
-  const unsigned grid = grid_for(npts, 128, 8);
+  const unsigned grid = pair_grid<K>(npts);
   KernF kf = make_kernf(f->kern);
   Scratch sc(s);
   const unsigned long long cap = (unsigned long long)std::min<int64_t>(npts, kBackwardRescueMax);
@@ -859,10 +801,10 @@ int launch_factor_backward_thread(graphgp_graph_t g, graphgp_factor_t f, int mod
   GGP_TRY(sc.alloc(&cnt, 1));
   GGP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
   const unsigned rgrid = (unsigned)num_sms() * 2;
-  constexpr size_t smem = ThreadStage<K>::kBytes;
+  constexpr size_t smem = PairLayout<K>::kBytes;
 #define GGP_FBT(KT)                                                                             \
-  GGP_CUDA(allow_dyn_smem(factor_backward_thread_kernel<K, KT>, smem));                         \
-  factor_backward_thread_kernel<K, KT><<<grid, kThreadBlock, smem, s>>>(                        \
+  GGP_CUDA(allow_dyn_smem(factor_backward_pair_kernel<K, KT>, smem));                         \
+  factor_backward_pair_kernel<K, KT><<<grid, kPairThreads, smem, s>>>(                        \
       g->xs, nbr, N, g->k, n0v, kf, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt, \
       cap);                                                                                     \
   factor_backward_rescue_kernel<K, KT><<<rgrid, 128, 0, s>>>(                                   \
@@ -885,7 +827,7 @@ int launch_nll_grad_fused(graphgp_graph_t g, const graphgp_kernel* kern, float n
                           cudaStream_t s) {
   const int64_t npts = g->N - g->n0;
   if (npts <= 0) return GRAPHGP_OK;
-  const unsigned grid = grid_for(npts, kThreadBlock, 8);
+  const unsigned grid = pair_grid<K>(npts);
   const KernF kf = make_kernf(*kern);
   Scratch sc(s);
   const unsigned long long cap = (unsigned long long)std::min<int64_t>(npts, kBackwardRescueMax);
@@ -895,10 +837,10 @@ int launch_nll_grad_fused(graphgp_graph_t g, const graphgp_kernel* kern, float n
   GGP_TRY(sc.alloc(&cnt, 1));
   GGP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
   const unsigned rgrid = (unsigned)num_sms() * 2;
-  constexpr size_t smem = fused_smem<K>();
+  constexpr size_t smem = PairLayout<K>::kBytes;
 #define GGP_NGF(KT)                                                                              \
   GGP_CUDA(allow_dyn_smem(nll_grad_fused_kernel<K, KT>, smem));                                  \
-  nll_grad_fused_kernel<K, KT><<<grid, kThreadBlock, smem, s>>>(                                 \
+  nll_grad_fused_kernel<K, KT><<<grid, kPairThreads, smem, s>>>(                                 \
       g->xs, g->nbr, g->N, g->k, g->n0, kf, nllbar, v, vbar, xi_tmp, xibar_tmp, thetabar, acc,  \
       not_pd, rows, cnt, cap);                                                                   \
   factor_backward_rescue_kernel<K, KT><<<rgrid, 128, 0, s>>>(                                    \
@@ -1000,10 +942,10 @@ int factor_backward_rows(graphgp_graph_t g, graphgp_factor_t f, int mode, const 
   const int32_t* nb = g->nbr + t0 * g->kp;
   const int64_t N = g->n0 + t1, n0v = g->n0 + t0;
   switch (g->kp) {
-    case 4: return launch_factor_backward_thread<4>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
-    case 8: return launch_factor_backward_thread<8>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
-    case 12: return launch_factor_backward_thread<12>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
-    case 16: return launch_factor_backward_thread<16>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
+    case 4: return launch_factor_backward_pair<4>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
+    case 8: return launch_factor_backward_pair<8>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
+    case 12: return launch_factor_backward_pair<12>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
+    case 16: return launch_factor_backward_pair<16>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
     case 20:
     case 24:
     case 28:

@@ -15,6 +15,7 @@
 // raised to that floor and counted.  logdet = sum log sigma_i^2 is reduced in
 // FP64 from the stored FP32 sigma (a running FP64 product with separate
 // exponent, one log per thread).
+#include "pointpair.cuh"
 #include "pointwide.cuh"
 
 namespace ggp {
@@ -114,53 +115,86 @@ __global__ void __launch_bounds__(128) point_factor_kernel(
   if (lane == 0 && clamped_rows) atomicAdd(not_pd, clamped_rows);
 }
 
-// One thread per point for k <= 16 (K = padded row length): the neighbour row
-// arrives as int4 loads, the k + 1 coordinates as float4 gathers, and the
-// whole factor stays in registers (point_factor_thread).  Same values as the
-// group kernel, bit for bit.
+// k <= 16 (K = padded row length): two lanes per point (pointpair.cuh).
 template <int K, int KT>
-__global__ void __launch_bounds__(128) point_factor_thread_kernel(
+__global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) point_factor_pair_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int64_t n0,
     KernF kf, float* __restrict__ b_out, float* __restrict__ sigma_out,
     double* __restrict__ logdet, unsigned long long* __restrict__ not_pd, RescueList rl) {
-  extern __shared__ __align__(16) unsigned char tstage[];
-  const ThreadStage<K> st(tstage);
-  double* W = reinterpret_cast<double*>(tstage + ThreadStage<K>::kBytes) +
-              (threadIdx.x >> 5) * (warp_rescue_bytes<K>() / sizeof(double));
+  using PL = PairLayout<K>;
+  extern __shared__ __align__(16) float psm[];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, r = lane & 1;
+  float* S = psm + (threadIdx.x >> 1) * PL::kStride;
   LogAcc acc;
   unsigned long long clamped_rows = 0;
   const int64_t npts = N - n0;
-  const int64_t total = (int64_t)gridDim.x * blockDim.x;
-  const int64_t iters = (npts + total - 1) / total;  // the same on every lane
-  for (int64_t it = 0; it < iters; it++) {
-    const int64_t t = it * total + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * PL::kPoints;
+  const int first = (threadIdx.x >> 5) * 16;
+  // the next point's indices and coordinates are loaded while this one's
+  // factor ends
+  PairLoad<K> ld;
+  float4 xn;
+  int64_t b0 = (int64_t)blockIdx.x * PL::kPoints;
+  auto at = [&](int64_t blk) { return min(blk + first + (lane >> 1), npts - 1); };
+  ld.indices(r, nbr + at(b0) * K);
+  ld.coords(r, xs);
+  xn = __ldg(xs + n0 + at(b0));
+  for (; b0 < npts; b0 += stride) {
+    // The block's warps start each point together: the straight-line code is
+    // longer than the instruction caches, and warps in step share its fetches
+    // (2^23 rows at K = 16: 3.65 -> 3.45 ms).
+    __syncthreads();
+    const int64_t base = b0 + first, t = base + (lane >> 1);
     const bool valid = t < npts;
     const int64_t i = n0 + (valid ? t : 0);
-    const int32_t* row = nbr + (valid ? t : 0) * K;
-    PointRegs<K> p;
-    const float4 xq = __ldg(xs + i);
-    bool deferred = false, rescue = false;
-    if (valid) {
-      stage_coords<K>(st, xs, row, k);
-      point_factor_thread<K, KT>(p, k, kf, st, xq);
-      if (needs_rescue(p, k, kf)) {
-        deferred = rl.defer(i);
-        rescue = !deferred;
+    const float4 xq = xn;
+    ld.stage(S, r);
+    PairFactor<K> f;
+    pair_factor<K, KT>(
+        f, S, r, k, kf, xq, [&] { ld.indices(r, nbr + at(b0 + stride) * K); },
+        [&] {
+          ld.coords(r, xs);
+          xn = __ldg(xs + n0 + at(b0 + stride));
+        });
+    bool rescue = valid && pair_needs_rescue(f, kf), deferred = false;
+    if (rescue && r == 0) deferred = rl.defer(i);
+    deferred = __shfl_sync(full, deferred, 0, 2);
+    if (valid && !rescue) {
+      float4* bo = reinterpret_cast<float4*>(b_out + t * K);
+#pragma unroll
+      for (int q = 0; q < (K + 4) / 8; q++) {
+        const int c0 = 2 * q, c1 = 2 * q + 1 < K / 4 ? 2 * q + 1 : 2 * q;
+        const float2 u = r ? f.b[2 * c1] : f.b[2 * c0], w = r ? f.b[2 * c1 + 1] : f.b[2 * c0 + 1];
+        if (2 * q + r < K / 4) bo[2 * q + r] = make_float4(u.x, u.y, w.x, w.y);
+      }
+      if (r == 0) {
+        sigma_out[i] = f.sigma;
+        acc.mul(f.sigma);
+        if (f.clamped) clamped_rows++;
       }
     }
-    warp_rescue<K, KT>(p, rescue, xs, row, k, xq, kf, W);  // list full: in place
-    if (!valid || deferred) continue;
-    float4* bo = reinterpret_cast<float4*>(b_out + t * K);
-#pragma unroll
-    for (int q = 0; q < K / 4; q++)
-      bo[q] = make_float4(p.y[4 * q], p.y[4 * q + 1], p.y[4 * q + 2], p.y[4 * q + 3]);
-    sigma_out[i] = p.sigma;
-    acc.mul(p.sigma);
-    if (p.clamped) clamped_rows++;
+    // the list is full: the warp recomputes such rows here, one at a time
+    unsigned m = __ballot_sync(full, rescue && !deferred && r == 0);
+    while (m) {
+      const int src = __ffs(m) - 1;
+      m &= m - 1;
+      __syncwarp();
+      const int64_t u = base + (src >> 1);
+      double* W = reinterpret_cast<double*>(psm + first * PL::kStride);
+      const WarpRow64 w = warp_row_factor64<K, KT>(xs, nbr + u * K, k, __ldg(xs + n0 + u), kf, W);
+      if (lane < K) b_out[u * K + lane] = lane < k ? (float)w.b : 0.0f;
+      if (lane == src) {
+        const float sg = (float)w.sigma;
+        sigma_out[i] = sg;
+        acc.mul(sg);
+        if (w.clamped) clamped_rows++;
+      }
+    }
   }
   block_add_double(acc.log_value(), logdet);
-  for (int o = 16; o; o >>= 1) clamped_rows += __shfl_xor_sync(0xffffffffu, clamped_rows, o);
-  if ((threadIdx.x & 31) == 0 && clamped_rows) atomicAdd(not_pd, clamped_rows);
+  for (int o = 16; o; o >>= 1) clamped_rows += __shfl_xor_sync(full, clamped_rows, o);
+  if (lane == 0 && clamped_rows) atomicAdd(not_pd, clamped_rows);
 }
 
 // 32 < k <= 64: one warp per point with the factor in shared memory
@@ -595,14 +629,14 @@ int launch_point(int type, graphgp_graph_t g, graphgp_factor_t f, const KernF& k
 }
 
 template <int K>
-int launch_point_thread(int type, graphgp_graph_t g, graphgp_factor_t f, const KernF& kf,
-                        const RescueList& rl, const RowView& rv, cudaStream_t s) {
+int launch_point_pair(int type, graphgp_graph_t g, graphgp_factor_t f, const KernF& kf,
+                      const RescueList& rl, const RowView& rv, cudaStream_t s) {
   const int64_t npts = rv.N - rv.n0;
-  const unsigned grid = grid_for(npts, kThreadBlock, 8);
-  constexpr size_t smem = ThreadStage<K>::kBytes + 4 * warp_rescue_bytes<K>();
+  const unsigned grid = pair_grid<K>(npts);
+  constexpr size_t smem = PairLayout<K>::kBytes;
 #define GGP_PT(KT)                                                                            \
-  GGP_CUDA(allow_dyn_smem(point_factor_thread_kernel<K, KT>, smem));                          \
-  point_factor_thread_kernel<K, KT><<<grid, kThreadBlock, smem, s>>>(                         \
+  GGP_CUDA(allow_dyn_smem(point_factor_pair_kernel<K, KT>, smem));                            \
+  point_factor_pair_kernel<K, KT><<<grid, kPairThreads, smem, s>>>(                           \
       g->xs, rv.nbr, rv.N, g->k, rv.n0, kf, rv.b, f->sigma, f->logdet, f->not_pd, rl)
   switch (type) {
     case GRAPHGP_MATERN12: GGP_PT(GRAPHGP_MATERN12); break;
@@ -653,10 +687,10 @@ int point_factor_rows(graphgp_graph_t g, graphgp_factor_t f, const KernF& kf, in
   GGP_TRY(sc.alloc(&rl.count, 1));
   GGP_CUDA(cudaMemsetAsync(rl.count, 0, sizeof(unsigned long long), s));
   switch (g->kp) {
-    case 4: GGP_TRY(launch_point_thread<4>(type, g, f, kf, rl, rv, s)); return launch_rescue<4>(type, g, f, kf, rl, rv, s);
-    case 8: GGP_TRY(launch_point_thread<8>(type, g, f, kf, rl, rv, s)); return launch_rescue<8>(type, g, f, kf, rl, rv, s);
-    case 12: GGP_TRY(launch_point_thread<12>(type, g, f, kf, rl, rv, s)); return launch_rescue<12>(type, g, f, kf, rl, rv, s);
-    case 16: GGP_TRY(launch_point_thread<16>(type, g, f, kf, rl, rv, s)); return launch_rescue<16>(type, g, f, kf, rl, rv, s);
+    case 4: GGP_TRY(launch_point_pair<4>(type, g, f, kf, rl, rv, s)); return launch_rescue<4>(type, g, f, kf, rl, rv, s);
+    case 8: GGP_TRY(launch_point_pair<8>(type, g, f, kf, rl, rv, s)); return launch_rescue<8>(type, g, f, kf, rl, rv, s);
+    case 12: GGP_TRY(launch_point_pair<12>(type, g, f, kf, rl, rv, s)); return launch_rescue<12>(type, g, f, kf, rl, rv, s);
+    case 16: GGP_TRY(launch_point_pair<16>(type, g, f, kf, rl, rv, s)); return launch_rescue<16>(type, g, f, kf, rl, rv, s);
     case 20:
     case 24:
     case 28:

@@ -5,7 +5,7 @@
 // of 2k + 5 with stored weights); this is the form for kernel parameters that
 // change at every step.
 //
-// Each thread owns one point and runs point_factor_thread (k <= 16; 16 < k
+// Two lanes own one point and run pair_factor (k <= 16; 16 < k
 // <= 32 in fused_group.cu) with the same FP64 rescue decision as the factor
 // kernel, so b and sigma are bit-identical to the stored factor's; the dot b . v_c then
 // follows the stored sweeps' summation order (the row cut into gen_lanes(K)
@@ -19,20 +19,10 @@
 // level l overlaps the end of level l - 1.  whiten: one grid-stride launch in
 // position order (no dependencies), optionally reducing xi.xi and
 // sum log sigma_i^2 in FP64.
-#include "pointfactor.cuh"
-#include "sweepsync.cuh"
+#include "pointpair.cuh"
 
 namespace ggp {
 namespace {
-
-template <int K, int KT>
-__device__ __forceinline__ void factor_at(PointRegs<K>& p, const ThreadStage<K>& st,
-                                          const float4* __restrict__ xs, const int32_t* row,
-                                          int64_t i, int k, const KernF& kf) {
-  const float4 xq = __ldg(xs + i);
-  stage_coords<K>(st, xs, row, k);
-  point_factor_thread<K, KT>(p, k, kf, st, xq);
-}
 
 __device__ inline void block_add_count(unsigned long long c, unsigned long long* out) {
   for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
@@ -40,35 +30,45 @@ __device__ inline void block_add_count(unsigned long long c, unsigned long long*
 }
 
 template <int K, int KT>
-__global__ void __launch_bounds__(128) whiten_fused_kernel(
+__global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) whiten_fused_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int64_t n0,
     KernF kf, const float* __restrict__ v, float* __restrict__ xi, double* __restrict__ sq,
     double* __restrict__ logdet, unsigned long long* __restrict__ not_pd) {
-  extern __shared__ __align__(16) unsigned char tstage[];
-  const ThreadStage<K> stg(tstage);
-  double* W = fused_rescue_ws<K>(tstage);
+  using PL = PairLayout<K>;
+  extern __shared__ __align__(16) float psm[];
+  const int lane = threadIdx.x & 31, r = lane & 1, first = (threadIdx.x >> 5) * 16;
+  float* S = psm + (threadIdx.x >> 1) * PL::kStride;
   const uint64_t pol_v = l2_evict_last();
   LogAcc lacc;
   double local = 0.0;
   unsigned long long clamped = 0;
   const int64_t npts = N - n0;
-  const int64_t total = (int64_t)gridDim.x * blockDim.x;
-  const int64_t iters = (npts + total - 1) / total;  // the same on every lane
-  for (int64_t it = 0; it < iters; it++) {
-    const int64_t t = it * total + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * PL::kPoints;
+  PairLoad<K> ld;
+  for (int64_t b0 = (int64_t)blockIdx.x * PL::kPoints; b0 < npts; b0 += stride) {
+    __syncthreads();  // the warps of a block share the instruction stream
+    const int64_t t = b0 + first + (lane >> 1);
     const bool valid = t < npts;
-    const int64_t i = n0 + (valid ? t : 0);
-    const int32_t* row = nbr + (valid ? t : 0) * K;
-    PointRegs<K> p;
-    if (valid) factor_at<K, KT>(p, stg, xs, row, i, k, kf);
-    warp_rescue<K, KT>(p, valid && needs_rescue(p, k, kf), xs, row, k, __ldg(xs + i), kf, W);
-    if (!valid) continue;
-    const float acc = dot_stored_order<K, false>(p.y, row, v, pol_v);
-    const float out = (ld_keep_f(v + i, pol_v) - acc) / p.sigma;
-    xi[i] = out;
-    local += (double)out * (double)out;
-    lacc.mul(p.sigma);
-    clamped += p.clamped ? 1 : 0;
+    const int64_t tt = valid ? t : npts - 1, i = n0 + tt;
+    const int32_t* row = nbr + tt * K;
+    const float4 xq = __ldg(xs + i);
+    ld.indices(r, row);
+    ld.coords(r, xs);
+    ld.stage(S, r);
+    PairFactor<K> f;
+    pair_factor<K, KT>(f, S, r, k, kf, xq);
+    float vv[K / 2];
+    pair_gather<K, false>(vv, r, row, v, pol_v);
+    pair_rescue<K, KT>(f, valid && pair_needs_rescue(f, kf), psm + first * PL::kStride, xs, row, k,
+                       xq, kf);
+    const float acc = pair_dot<K>(f.b, vv, r);
+    if (valid && r == 0) {
+      const float out = (ld_keep_f(v + i, pol_v) - acc) / f.sigma;
+      xi[i] = out;
+      local += (double)out * (double)out;
+      lacc.mul(f.sigma);
+      clamped += f.clamped ? 1 : 0;
+    }
   }
   if (sq) block_add_double(local, sq);
   if (logdet) block_add_double(lacc.log_value(), logdet);
@@ -76,37 +76,46 @@ __global__ void __launch_bounds__(128) whiten_fused_kernel(
 }
 
 template <int K, int KT>
-__global__ void __launch_bounds__(128) generate_fused_kernel(
+__global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) generate_fused_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int k, int64_t n0, KernF kf,
     const float* __restrict__ xi, float* v, const int64_t* __restrict__ level_off,
     int num_levels, LevelBarrier lb, unsigned long long* __restrict__ not_pd) {
+  using PL = PairLayout<K>;
   __shared__ int s_flag;
-  extern __shared__ __align__(16) unsigned char tstage[];
-  const ThreadStage<K> stg(tstage);
-  double* W = fused_rescue_ws<K>(tstage);
+  extern __shared__ __align__(16) float psm[];
+  const int lane = threadIdx.x & 31, r = lane & 1, first = (threadIdx.x >> 5) * 16;
+  float* S = psm + (threadIdx.x >> 1) * PL::kStride;
   const uint64_t pol_v = l2_evict_last();
   unsigned long long clamped = 0;
+  PairLoad<K> ld;
   for (int l = 1; l < num_levels; l++) {
     const int64_t lo = level_off[l], n = level_off[l + 1] - lo;
     const int64_t per = (n + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = lo + min((int64_t)blockIdx.x * per, n);
     const int64_t hi = lo + min((int64_t)(blockIdx.x + 1) * per, n);
-    const int64_t steps = (hi - b0 + blockDim.x - 1) / blockDim.x;
+    const int64_t steps = (hi - b0 + PL::kPoints - 1) / PL::kPoints;
     if (steps == 0 && l > 1 && lb.wait(l - 1, gridDim.x, &s_flag)) return;
     for (int64_t st = 0; st < steps; st++) {
-      const int64_t q = b0 + st * blockDim.x + threadIdx.x;
+      const int64_t q = b0 + st * PL::kPoints + first + (lane >> 1);
       const bool active = q < hi;
-      const int32_t* row = nbr + (active ? q - n0 : 0) * K;
-      PointRegs<K> p;
-      if (active) factor_at<K, KT>(p, stg, xs, row, q, k, kf);
-      warp_rescue<K, KT>(p, active && needs_rescue(p, k, kf), xs, row, k,
-                         __ldg(xs + (active ? q : n0)), kf, W);
+      const int64_t qq = active ? q : hi - 1;
+      const int32_t* row = nbr + (qq - n0) * K;
+      const float4 xq = __ldg(xs + qq);
+      ld.indices(r, row);
+      ld.coords(r, xs);
+      ld.stage(S, r);
+      PairFactor<K> f;
+      pair_factor<K, KT>(f, S, r, k, kf, xq);
+      pair_rescue<K, KT>(f, active && pair_needs_rescue(f, kf), psm + first * PL::kStride, xs, row,
+                         k, xq, kf);
       // the level's inputs are complete once every block arrived at l - 1
       if (st == 0 && l > 1 && lb.wait(l - 1, gridDim.x, &s_flag)) return;
-      if (active) {
-        const float acc = dot_stored_order<K, true>(p.y, row, v, pol_v);
-        st_keep_f(v + q, fmaf(p.sigma, xi[q], acc), pol_v);
-        clamped += p.clamped ? 1 : 0;
+      float vv[K / 2];
+      pair_gather<K, true>(vv, r, row, v, pol_v);
+      const float acc = pair_dot<K>(f.b, vv, r);
+      if (active && r == 0) {
+        st_keep_f(v + q, fmaf(f.sigma, xi[q], acc), pol_v);
+        clamped += f.clamped ? 1 : 0;
       }
     }
     __syncthreads();
@@ -151,11 +160,11 @@ int launch_whiten_fused(graphgp_graph_t g, int type, const KernF& kf, const floa
                         double* sq, double* logdet, unsigned long long* not_pd, cudaStream_t s) {
   const int64_t npts = g->N - g->n0;
   if (npts <= 0) return GRAPHGP_OK;
-  const unsigned grid = grid_for(npts, kThreadBlock, 8);
-  constexpr size_t smem = fused_smem<K>();
+  const unsigned grid = pair_grid<K>(npts);
+  constexpr size_t smem = PairLayout<K>::kBytes;
 #define GGP_WF(KT)                                                                            \
   GGP_CUDA(allow_dyn_smem(whiten_fused_kernel<K, KT>, smem));                                 \
-  whiten_fused_kernel<K, KT><<<grid, kThreadBlock, smem, s>>>(g->xs, g->nbr, g->N, g->k, g->n0, \
+  whiten_fused_kernel<K, KT><<<grid, kPairThreads, smem, s>>>(g->xs, g->nbr, g->N, g->k, g->n0, \
                                                               kf, v, xi, sq, logdet, not_pd)
   switch (type) {
     case GRAPHGP_MATERN12: GGP_WF(GRAPHGP_MATERN12); break;
@@ -171,11 +180,11 @@ int launch_whiten_fused(graphgp_graph_t g, int type, const KernF& kf, const floa
 template <int K, int KT>
 int launch_generate_fused_kt(graphgp_graph_t g, const KernF& kf, const float* xi, float* v,
                              unsigned long long* not_pd, cudaStream_t s) {
-  constexpr size_t smem = fused_smem<K>();
+  constexpr size_t smem = PairLayout<K>::kBytes;
   GGP_CUDA(allow_dyn_smem(generate_fused_kernel<K, KT>, smem));
   static int max_grid_dev[kMaxDevices] = {};
-  const int max_grid = coop_grid_cached(max_grid_dev, generate_fused_kernel<K, KT>, kThreadBlock, smem);
-  const int64_t want = (g->max_level_size + 127) / 128;
+  const int max_grid = coop_grid_cached(max_grid_dev, generate_fused_kernel<K, KT>, kPairThreads, smem);
+  const int64_t want = (g->max_level_size + PairLayout<K>::kPoints - 1) / PairLayout<K>::kPoints;
   const int grid = (int)std::min<int64_t>(max_grid, std::max<int64_t>(want, 1));
   GGP_CUDA(cudaMemsetAsync(g->level_bar, 0, g->num_levels * sizeof(uint32_t), s));
   LevelBarrier lb{g->level_bar, g->err, g->max_spin};
@@ -188,7 +197,7 @@ int launch_generate_fused_kt(graphgp_graph_t g, const KernF& kf, const float* xi
   void* args[] = {(void*)&xs, (void*)&nbr, (void*)&k, (void*)&n0, (void*)&kf, (void*)&xi,
                   (void*)&v,  (void*)&lo,  (void*)&nl, (void*)&lb, (void*)&not_pd};
   GGP_CUDA(cudaLaunchCooperativeKernel((const void*)generate_fused_kernel<K, KT>, dim3(grid),
-                                       dim3(kThreadBlock), args, smem, s));
+                                       dim3(kPairThreads), args, smem, s));
   return GRAPHGP_OK;
 }
 

@@ -194,8 +194,8 @@ __device__ __forceinline__ void point_factor_group(PointState<G>& st, int a, int
       piv = pfloor;
       st.clamped = true;
     }
-    float ljj = sqrtf(piv);
-    float inv = 1.0f / ljj;
+    float ljj = sqrt_newton(piv);
+    float inv = rcp_newton(ljj);
     st.max_ratio = fmaxf(st.max_ratio, mjj * inv * inv);
     float laj = (a == j) ? ljj : tv * inv;
     st.A[j] = laj;
@@ -263,309 +263,12 @@ __device__ __forceinline__ float group_chol_solve(const PointState<G>& st, int a
   return g_own;
 }
 
-
-
-// ---- one thread per point (k <= 16) ----------------------------------------
-// The same arithmetic as point_factor_group, element by element and in the
-// same order, but with the whole lower triangle of L in one thread's
-// registers: no shuffles, no shared memory, each variogram value evaluated
-// once (the group form evaluates every row in full on its lanes).  K is the padded
-// row length (4, 8, 12 or 16); entries a >= k are identity padding, which
-// passes through every step without changing the real entries (unit pivot,
-// zero off-diagonal, zero right-hand side), so all loops run K steps.  The
-// column loops are unrolled at compile time (static_for) so that every
-// register-array index is a constant.
-
-__host__ __device__ constexpr int tri(int a, int c) { return a * (a + 1) / 2 + c; }
-
 template <int I, int N, class F>
 __device__ __forceinline__ void static_for(F&& f) {
   if constexpr (I < N) {
     f(std::integral_constant<int, I>{});
     static_for<I + 1, N>(f);
   }
-}
-
-template <int K>
-struct PointRegs {
-  float L[K * (K + 1) / 2];  // M, then L = chol(M): L[tri(a, c)], c <= a
-  float y[K];                // m, y = L^-1 m, beta = L^-T y, then b (zero for a >= k)
-  float sigma;
-  bool clamped;
-  float max_ratio;           // max_j M_jj / pivot_j
-  float varw;                // Var(w)
-  bool inc;                  // increment form
-  // 1 / L_jj, recomputed where needed (the same correctly rounded quotient)
-  __device__ __forceinline__ float inv(int j) const { return 1.0f / L[tri(j, j)]; }
-};
-
-// Schur value t = K_aj - sum_{m<j} L_am L_jm with the group form's two
-// accumulators (m = 0, 2 mod 4 and m = 1, 3 mod 4 over whole blocks of four).
-template <int K, int J, int A>
-__device__ __forceinline__ float schur_value(const PointRegs<K>& p) {
-  float tv = p.L[tri(A, J)];
-  float t2 = 0.0f;
-#pragma unroll
-  for (int m = 0; m + 4 <= J; m += 4) {
-    tv = fmaf(-p.L[tri(A, m)], p.L[tri(J, m)], tv);
-    t2 = fmaf(-p.L[tri(A, m + 1)], p.L[tri(J, m + 1)], t2);
-    tv = fmaf(-p.L[tri(A, m + 2)], p.L[tri(J, m + 2)], tv);
-    t2 = fmaf(-p.L[tri(A, m + 3)], p.L[tri(J, m + 3)], t2);
-  }
-#pragma unroll
-  for (int m = (J / 4) * 4; m < J; m++) tv = fmaf(-p.L[tri(A, m)], p.L[tri(J, m)], tv);
-  return tv + t2;
-}
-
-// Shared-memory staging of the one-thread-per-point kernels (blocks of
-// kThreadBlock threads).  Evaluating the kernel values of a conditional
-// fully unrolled, with the whole factor live in registers, made the code
-// larger than the instruction cache (ncu: "no instruction" was the largest
-// stall).  The thread instead stages its k neighbour coordinates and then
-// its k(k-1)/2 + k kernel values in shared memory in a rolled loop, and the
-// unrolled factor reads them back.  Entry e of thread t sits at
-// [e * kThreadBlock + t] (consecutive threads, consecutive words).
-constexpr int kThreadBlock = 128;
-
-template <int K>
-struct ThreadStage {
-  static constexpr int kPairs = K * (K - 1) / 2;            // (a, c), c < a
-  static constexpr int kEntries = kPairs + K;                // and (a, i)
-  static constexpr size_t kBytes = (size_t)kThreadBlock * (16 * K + 4 * kEntries);
-  float4* X;  // neighbour coordinates, X[a * kThreadBlock]
-  float* E;   // kernel values, E[e * kThreadBlock]
-  __device__ __forceinline__ ThreadStage(unsigned char* smem) {
-    X = reinterpret_cast<float4*>(smem) + threadIdx.x;
-    E = reinterpret_cast<float*>(smem + (size_t)16 * K * kThreadBlock) + threadIdx.x;
-  }
-};
-
-__host__ __device__ constexpr int pair_ix(int a, int c) { return a * (a - 1) / 2 + c; }
-
-// Loads the k neighbour coordinates of a row (int4 index loads, float4
-// gathers) into the stage; entries k..K-1 are not written.
-template <int K>
-__device__ __forceinline__ void stage_coords(const ThreadStage<K>& st,
-                                             const float4* __restrict__ xs,
-                                             const int32_t* __restrict__ row, int k) {
-#pragma unroll
-  for (int q = 0; q < K / 4; q++) {
-    if (4 * q >= k) break;
-    const int4 c = __ldg(reinterpret_cast<const int4*>(row) + q);
-    st.X[(4 * q) * kThreadBlock] = __ldg(xs + c.x);
-    if (4 * q + 1 < k) st.X[(4 * q + 1) * kThreadBlock] = __ldg(xs + c.y);
-    if (4 * q + 2 < k) st.X[(4 * q + 2) * kThreadBlock] = __ldg(xs + c.z);
-    if (4 * q + 3 < k) st.X[(4 * q + 3) * kThreadBlock] = __ldg(xs + c.w);
-  }
-}
-
-// The factor of the row whose coordinates stage_coords put in `st`.
-template <int K, int KT>
-__device__ __forceinline__ void point_factor_thread(PointRegs<K>& p, int k, const KernF& kf,
-                                                    const ThreadStage<K>& st, float4 xq) {
-  const float k0 = kf.s2 + kf.nug;
-  const float nug = kf.nug;
-  const KG q0 = kappa_gamma_d2<KT>(kf, sqdist(st.X[0], xq));
-  const bool inc = q0.g < 0.5f * kf.s2;
-  p.inc = inc;
-  // gamma (increment form) or kappa (covariance form) of every pair and of
-  // every neighbour with the point, in a rolled loop taking four pairs per
-  // iteration: their coordinates are read before any value is stored, so
-  // the four evaluations overlap
-#pragma unroll 1
-  for (int a = 1; a < k; a++) {
-    const float4 xa = st.X[a * kThreadBlock];
-    float* ea = st.E + pair_ix(a, 0) * kThreadBlock;
-    int c = 0;
-#pragma unroll 1
-    for (; c + 4 <= a; c += 4) {
-      float4 xc[4];
-#pragma unroll
-      for (int u = 0; u < 4; u++) xc[u] = st.X[(c + u) * kThreadBlock];
-      float e[4];
-#pragma unroll
-      for (int u = 0; u < 4; u++) {
-        const KG kg = kappa_gamma_d2<KT>(kf, sqdist(xa, xc[u]));
-        e[u] = inc ? kg.g : kg.k;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; u++) ea[(c + u) * kThreadBlock] = e[u];
-    }
-#pragma unroll 1
-    for (; c < a; c++) {
-      const KG kg = kappa_gamma_d2<KT>(kf, sqdist(xa, st.X[c * kThreadBlock]));
-      ea[c * kThreadBlock] = inc ? kg.g : kg.k;
-    }
-    const KG kq = kappa_gamma_d2<KT>(kf, sqdist(xa, xq));
-    st.E[(ThreadStage<K>::kPairs + a) * kThreadBlock] = inc ? kq.g : kq.k;
-  }
-  // into registers; padding rows and columns (a >= k) are zero
-  static_for<1, K>([&](auto Ar) {
-    constexpr int a = decltype(Ar)::value;
-    const bool real = a < k;
-#pragma unroll
-    for (int c = 0; c < a; c++) p.L[tri(a, c)] = real ? st.E[pair_ix(a, c) * kThreadBlock] : 0.0f;
-    p.y[a] = real ? st.E[(ThreadStage<K>::kPairs + a) * kThreadBlock] : 0.0f;
-  });
-  p.y[0] = inc ? q0.g : q0.k;
-  // M and m (column 0 last: in the increment form its entries are g_a0)
-  const float e0i = p.y[0];
-  static_for<1, K>([&](auto Ac) {
-    constexpr int a = decltype(Ac)::value;
-    const bool real = a < k;
-    const float ea0 = p.L[tri(a, 0)];
-#pragma unroll
-    for (int c = 1; c < a; c++)
-      p.L[tri(a, c)] = real ? (inc ? ((ea0 + p.L[tri(c, 0)]) - p.L[tri(a, c)]) + nug : p.L[tri(a, c)])
-                            : 0.0f;
-    p.L[tri(a, a)] = real ? (inc ? 2.0f * (ea0 + nug) : k0) : 1.0f;
-    p.y[a] = real ? (inc ? ((ea0 + e0i) - p.y[a]) + nug : p.y[a]) : 0.0f;
-  });
-#pragma unroll
-  for (int a = 1; a < K; a++)
-    p.L[tri(a, 0)] = a < k ? (inc ? -(p.L[tri(a, 0)] + nug) : p.L[tri(a, 0)]) : 0.0f;
-  p.L[tri(0, 0)] = k0;
-  p.y[0] = inc ? -(e0i + nug) : e0i;
-  p.varw = inc ? 2.0f * (e0i + nug) : k0;
-  DF s2{p.varw, 0.0f};
-  bool clamped = false;
-  float max_ratio = 1.0f;
-  const float pfloor = kPdFloor * k0;
-  static_for<0, K>([&](auto Jc) {
-    constexpr int j = decltype(Jc)::value;
-    const float mjj = p.L[tri(j, j)];
-    float piv = schur_value<K, j, j>(p);
-    if (!(piv > pfloor)) {
-      piv = pfloor;
-      clamped = true;
-    }
-    const float ljj = sqrtf(piv);
-    const float inv = 1.0f / ljj;
-    max_ratio = fmaxf(max_ratio, mjj * inv * inv);  // padding: 1
-    static_for<j + 1, K>([&](auto Ac) {
-      constexpr int a = decltype(Ac)::value;
-      p.L[tri(a, j)] = schur_value<K, j, a>(p) * inv;
-    });
-    p.L[tri(j, j)] = ljj;
-    const float yj = p.y[j] * inv;
-    p.y[j] = yj;
-#pragma unroll
-    for (int a = j + 1; a < K; a++) p.y[a] = fmaf(-p.L[tri(a, j)], yj, p.y[a]);
-    s2 = df_sub_square(s2, yj);
-  });
-  float sig2 = s2.hi + s2.lo;
-  if (!(sig2 > pfloor)) {
-    sig2 = pfloor;
-    clamped = true;
-  }
-  p.clamped = clamped;
-  p.max_ratio = max_ratio;
-  p.sigma = sqrtf(sig2);
-  // beta = L^-T y, last entry first
-  static_for<0, K>([&](auto Jr) {
-    constexpr int j = K - 1 - decltype(Jr)::value;
-    const float bj = p.y[j] * p.inv(j);
-    p.y[j] = bj;
-#pragma unroll
-    for (int a = 0; a < j; a++) p.y[a] = fmaf(-p.L[tri(j, a)], bj, p.y[a]);
-  });
-  // increment form: b_0 = 1 + beta_0 - sum_{a>=1} beta_a (padding entries are zero)
-  float sb = 0.0f;
-#pragma unroll
-  for (int a = 1; a < K; a++) sb += p.y[a];
-  if (inc) p.y[0] = (1.0f + p.y[0]) - sb;
-}
-
-// Solves K_cc g = r in place with the factor of point_factor_thread
-// (g = T^T M^-1 T r, same operation order as group_chol_solve); r must be
-// zero at padding entries.
-template <int K>
-__device__ __forceinline__ void thread_chol_solve(const PointRegs<K>& p, int k, float (&r)[K]) {
-#pragma unroll
-  for (int a = 1; a < K; a++)
-    if (p.inc && a < k) r[a] -= r[0];
-  static_for<0, K>([&](auto Jc) {
-    constexpr int j = decltype(Jc)::value;
-    const float zj = r[j] * p.inv(j);
-    r[j] = zj;
-#pragma unroll
-    for (int a = j + 1; a < K; a++) r[a] = fmaf(-p.L[tri(a, j)], zj, r[a]);
-  });
-  static_for<0, K>([&](auto Jr) {
-    constexpr int j = K - 1 - decltype(Jr)::value;
-    const float gj = r[j] * p.inv(j);
-    r[j] = gj;
-#pragma unroll
-    for (int a = 0; a < j; a++) r[a] = fmaf(-p.L[tri(j, a)], gj, r[a]);
-  });
-  float sg = 0.0f;
-#pragma unroll
-  for (int a = 1; a < K; a++) sg += r[a];
-  if (p.inc) r[0] -= sg;
-}
-
-// Whether a conditional computed in FP32 must be recomputed in FP64 (see
-// rescue.cuh): a floored pivot or sigma^2, a row-error estimate above the
-// kernel's threshold, or a non-finite weight or sigma.
-template <int K>
-__device__ __forceinline__ bool needs_rescue(const PointRegs<K>& p, int k, const KernF& kf) {
-  bool bad = p.clamped || row_error_too_large(p.max_ratio, p.varw, p.sigma, kf) ||
-             !isfinite(p.sigma);
-#pragma unroll
-  for (int a = 0; a < K; a++) bad |= !isfinite(p.y[a]);
-  return bad;
-}
-
-// Shared memory of the warp-cooperative FP64 rescue (rescue.cuh) for one warp
-// of a one-thread-per-point kernel: K (K + 1) doubles.
-template <int K>
-__host__ __device__ constexpr size_t warp_rescue_bytes() { return (size_t)K * (K + 1) * sizeof(double); }
-
-// The rows of the warp's lanes with `need` set are recomputed in FP64, one
-// row at a time by the whole warp (warp_row_factor64); each such lane
-// receives its b (zero past k), sigma and floor flag, rounded to FP32.  Every
-// lane of the warp must call this (a collective); W is the warp's shared
-// memory of warp_rescue_bytes<K>().
-template <int K, int KT>
-__device__ __forceinline__ void warp_rescue(PointRegs<K>& p, bool need,
-                                            const float4* __restrict__ xs, const int32_t* row,
-                                            int k, float4 xq, const KernF& kf, double* W) {
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  unsigned m = __ballot_sync(full, need);
-  while (m) {
-    const int src = __ffs(m) - 1;
-    m &= m - 1;
-    const int32_t* r = reinterpret_cast<const int32_t*>(
-        __shfl_sync(full, reinterpret_cast<unsigned long long>(row), src));
-    float4 q;
-    q.x = __shfl_sync(full, xq.x, src);
-    q.y = __shfl_sync(full, xq.y, src);
-    q.z = __shfl_sync(full, xq.z, src);
-    q.w = 0.0f;
-    const WarpRow64 w = warp_row_factor64<K, KT>(xs, r, k, q, kf, W);
-    float* bf = reinterpret_cast<float*>(W);
-    bf[lane] = (float)w.b;
-    __syncwarp();
-    if (lane == src) {
-#pragma unroll
-      for (int a = 0; a < K; a++) p.y[a] = a < k ? bf[a] : 0.0f;
-      p.sigma = (float)w.sigma;
-      p.clamped = w.clamped;
-    }
-    __syncwarp();
-  }
-}
-
-// Dynamic shared memory of the one-thread-per-point fused kernels: the
-// staging area, then each warp's FP64 rescue workspace.
-template <int K>
-constexpr size_t fused_smem() { return ThreadStage<K>::kBytes + 4 * warp_rescue_bytes<K>(); }
-
-template <int K>
-__device__ __forceinline__ double* fused_rescue_ws(unsigned char* smem) {
-  return reinterpret_cast<double*>(smem + ThreadStage<K>::kBytes) +
-         (threadIdx.x >> 5) * (warp_rescue_bytes<K>() / sizeof(double));
 }
 
 }  // namespace ggp

@@ -98,8 +98,8 @@ __device__ __forceinline__ WideFactor point_factor_wide(WideWarp& W, int k, cons
       piv = pfloor;
       r.clamped = true;
     }
-    const float ljj = sqrtf(piv);
-    const float inv = 1.0f / ljj;
+    const float ljj = sqrt_newton(piv);
+    const float inv = rcp_newton(ljj);
     r.max_ratio = fmaxf(r.max_ratio, W.g[j] * inv * inv);
     const float yj = W.y[j] * inv;
     s2 = df_sub_square(s2, yj);
@@ -137,7 +137,7 @@ __device__ __forceinline__ WideFactor point_factor_wide(WideWarp& W, int k, cons
   r.sigma = sqrtf(sig2);
   // beta = L^-T y, last entry first
   for (int j = k - 1; j >= 0; j--) {
-    const float bj = W.y[j] * (1.0f / W.L[j * kWideLd + j]);
+    const float bj = W.y[j] * rcp_newton(W.L[j * kWideLd + j]);
     __syncwarp();
     for (int a = lane; a < j; a += 32) W.y[a] = fmaf(-W.L[j * kWideLd + a], bj, W.y[a]);
     if (lane == 0) W.y[j] = bj;
@@ -164,14 +164,14 @@ __device__ __forceinline__ void wide_chol_solve(WideWarp& W, int k, bool inc) {
     __syncwarp();
   }
   for (int j = 0; j < k; j++) {
-    const float zj = W.g[j] * (1.0f / W.L[j * kWideLd + j]);
+    const float zj = W.g[j] * rcp_newton(W.L[j * kWideLd + j]);
     __syncwarp();
     for (int a = j + 1 + lane; a < k; a += 32) W.g[a] = fmaf(-W.L[a * kWideLd + j], zj, W.g[a]);
     if (lane == 0) W.g[j] = zj;
     __syncwarp();
   }
   for (int j = k - 1; j >= 0; j--) {
-    const float gj = W.g[j] * (1.0f / W.L[j * kWideLd + j]);
+    const float gj = W.g[j] * rcp_newton(W.L[j * kWideLd + j]);
     __syncwarp();
     for (int a = lane; a < j; a += 32) W.g[a] = fmaf(-W.L[j * kWideLd + a], gj, W.g[a]);
     if (lane == 0) W.g[j] = gj;

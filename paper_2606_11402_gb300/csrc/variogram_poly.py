@@ -73,6 +73,15 @@ def emit(name, f, lo, hi, deg, doc):
     print("  return h;")
     print("}")
     print()
+    print(f"// {name} of two arguments (packed FP32)")
+    print(f"__device__ __forceinline__ float2 {name}_2(float2 x) {{")
+    print(f"  constexpr float c[{deg + 1}] = {{{body}}};")
+    print(f"  float2 h = make_float2(c[{deg}], c[{deg}]);")
+    print("#pragma unroll")
+    print(f"  for (int i = {deg - 1}; i >= 0; i--) h = __ffma2_rn(h, x, make_float2(c[i], c[i]));")
+    print("  return h;")
+    print("}")
+    print()
 
 
 if __name__ == "__main__":
