@@ -1,6 +1,5 @@
-// Per-point conditioning factors (Sec. 2.1 Eq. 2; Alg. 1) and the dense
-// initial block (the dense initial batch of Alg. 1; Sec. 2.2 "Batch
-// construction").
+// Per-point conditioning factors (Sec. 2.1 Eq. 2; Alg. 1).  The dense initial
+// block is in dense.cu.
 //
 // Per point i with c = c(i): b_i = K_ic K_cc^-1 and sigma_i^2 =
 // K_ii - K_ic K_cc^-1 K_ci.  A group of G lanes (G = 8, 16 or 32 >= k) of one
@@ -330,279 +329,6 @@ int launch_rescue(int type, graphgp_graph_t g, graphgp_factor_t f, const KernF& 
   return GRAPHGP_OK;
 }
 
-// What the FP32 dense factor leaves for dense_finish_kernel.
-struct DenseCheck {
-  double logdet;           // sum log L0_ii^2 of the FP32 block
-  unsigned long long bad;  // floored pivots
-  float min_piv;           // smallest pivot before flooring
-};
-
-// Dense block: K_00 (lower triangle) in global memory.
-template <int KT>
-__global__ void dense_fill_kernel(const float4* __restrict__ xs, int n0, KernF kf,
-                                  float* __restrict__ A) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)n0 * n0;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int i = (int)(e / n0), j = (int)(e % n0);
-    float v = 0.0f;
-    if (j < i) v = kappa_d2<KT>(kf, sqdist(xs[i], xs[j]));
-    else if (j == i) v = kf.s2 + kf.nug;
-    A[e] = v;
-  }
-}
-
-// One block, left-looking Cholesky by columns on the n0 x n0 matrix in
-// global memory (L2-resident), with the pivot floor; then L0^-1 column by
-// column; sigma_i = L0_ii; adds sum log L0_ii^2 to logdet.
-__global__ void __launch_bounds__(1024) dense_chol_kernel(float* __restrict__ A,
-                                                          float* __restrict__ W, int n0,
-                                                          float* __restrict__ sigma,
-                                                          DenseCheck* __restrict__ chk) {
-  extern __shared__ float rowj[];  // [n0]
-  __shared__ float s_inv;
-  __shared__ unsigned long long s_bad;
-  __shared__ float s_minpiv;
-  if (threadIdx.x == 0) {
-    s_bad = 0;
-    s_minpiv = A[0];
-  }
-  const float k0 = A[0];
-  for (int j = 0; j < n0; j++) {
-    for (int m = threadIdx.x; m < j; m += blockDim.x) rowj[m] = A[(int64_t)j * n0 + m];
-    __syncthreads();
-    for (int r = j + threadIdx.x; r < n0; r += blockDim.x) {
-      const float* ar = A + (int64_t)r * n0;
-      float t0 = ar[j], t1 = 0.0f;
-      int m = 0;
-      for (; m + 1 < j; m += 2) {
-        t0 = fmaf(-ar[m], rowj[m], t0);
-        t1 = fmaf(-ar[m + 1], rowj[m + 1], t1);
-      }
-      if (m < j) t0 = fmaf(-ar[m], rowj[m], t0);
-      float tv = t0 + t1;
-      if (r == j) {
-        float fl = kPdFloor * k0;
-        s_minpiv = fminf(s_minpiv, tv);
-        if (!(tv > fl)) {
-          tv = fl;
-          s_bad++;
-        }
-        float l = sqrtf(tv);
-        A[(int64_t)j * n0 + j] = l;
-        s_inv = 1.0f / l;
-      } else {
-        rowj[n0 - 1 - (r - j - 1)] = tv;  // park in the unused tail of rowj
-      }
-    }
-    __syncthreads();
-    float inv = s_inv;
-    for (int r = j + 1 + threadIdx.x; r < n0; r += blockDim.x)
-      A[(int64_t)r * n0 + j] = rowj[n0 - 1 - (r - j - 1)] * inv;
-    __syncthreads();
-  }
-  // inverse: column c solves L w = e_c
-  for (int c = threadIdx.x; c < n0; c += blockDim.x) {
-    for (int i = 0; i < c; i++) W[(int64_t)i * n0 + c] = 0.0f;
-    W[(int64_t)c * n0 + c] = 1.0f / A[(int64_t)c * n0 + c];
-    for (int i = c + 1; i < n0; i++) {
-      const float* ar = A + (int64_t)i * n0;
-      float t = 0.0f;
-      for (int m = c; m < i; m++) t = fmaf(ar[m], W[(int64_t)m * n0 + c], t);
-      W[(int64_t)i * n0 + c] = -t / ar[i];
-    }
-  }
-  __syncthreads();
-  double lsum = 0.0;
-  for (int i = threadIdx.x; i < n0; i += blockDim.x) {
-    float l = A[(int64_t)i * n0 + i];
-    sigma[i] = l;
-    lsum += log((double)l * (double)l);
-  }
-  block_add_double(lsum, &chk->logdet);
-  if (threadIdx.x == 0) {
-    chk->bad = s_bad;
-    chk->min_piv = s_minpiv;
-  }
-}
-
-// Dense block with the lower triangle held in shared memory (n0 <= 320): one
-// block of 1024 threads, four threads per row for every dot product.
-//   Cholesky, left-looking by columns: t_r = A_rj - sum_{m<j} L_rm L_jm for
-//   r >= j, pivot t_j (floored at 1e-7 K_00 and counted), L_rj = t_r / L_jj.
-//   Inverse in place, last column first: with the trailing block already
-//   inverted (W2), column j of W = L^-1 is W_jj = 1 / L_jj and
-//   W_rj = -W_jj sum_{j<m<=r} W2_rm L_mj for r > j.
-// Outputs as dense_chol_kernel: L0 and L0^-1 row-major with zero upper part,
-// sigma_i = L0_ii, logdet += sum log L0_ii^2 (FP64), not-PD count.
-constexpr int kDenseSmemMax = 320;
-__device__ __forceinline__ int tri_ix(int r, int c) { return r * (r + 1) / 2 + c; }
-
-__global__ void __launch_bounds__(1024) dense_chol_smem_kernel(float* __restrict__ A,
-                                                               float* __restrict__ W, int n0,
-                                                               float* __restrict__ sigma,
-                                                               DenseCheck* __restrict__ chk) {
-  extern __shared__ float S[];         // [tri(n0)] packed lower triangle
-  float* tr = S + n0 * (n0 + 1) / 2;   // [n0] column values of one step
-  __shared__ unsigned long long s_bad;
-  __shared__ float s_minpiv;
-  const int w = threadIdx.x >> 2, part = threadIdx.x & 3;
-  if (threadIdx.x == 0) {
-    s_bad = 0;
-    s_minpiv = A[0];
-  }
-  for (int e = threadIdx.x; e < n0 * n0; e += blockDim.x) {
-    const int r = e / n0, c = e - r * n0;
-    if (c <= r) S[tri_ix(r, c)] = A[e];
-  }
-  __syncthreads();
-  const float fl = kPdFloor * S[0];
-  for (int j = 0; j < n0; j++) {
-    const float* Lj = S + tri_ix(j, 0);
-    for (int r0 = 0; r0 < n0; r0 += 256) {
-      const int r = r0 + w;
-      float acc = 0.0f;
-      if (r >= j && r < n0) {
-        const float* Lr = S + tri_ix(r, 0);
-        for (int m = part; m < j; m += 4) acc = fmaf(Lr[m], Lj[m], acc);
-      }
-      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-      acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-      if (part == 0 && r >= j && r < n0) tr[r] = S[tri_ix(r, j)] - acc;
-    }
-    __syncthreads();
-    float piv = tr[j];
-    const bool bad = !(piv > fl);
-    if (bad) piv = fl;
-    const float ljj = sqrtf(piv);
-    const float inv = 1.0f / ljj;
-    for (int r = j + 1 + threadIdx.x; r < n0; r += blockDim.x) S[tri_ix(r, j)] = tr[r] * inv;
-    if (threadIdx.x == 0) {
-      S[tri_ix(j, j)] = ljj;
-      s_minpiv = fminf(s_minpiv, tr[j]);
-      if (bad) s_bad++;
-    }
-    __syncthreads();
-  }
-  double lsum = 0.0;
-  for (int e = threadIdx.x; e < n0 * n0; e += blockDim.x) {
-    const int r = e / n0, c = e - r * n0;
-    A[e] = c <= r ? S[tri_ix(r, c)] : 0.0f;
-  }
-  for (int i = threadIdx.x; i < n0; i += blockDim.x) {
-    const float l = S[tri_ix(i, i)];
-    sigma[i] = l;
-    lsum += log((double)l * (double)l);
-  }
-  __syncthreads();
-  for (int j = n0 - 1; j >= 0; j--) {
-    const float d = 1.0f / S[tri_ix(j, j)];
-    for (int r0 = 0; r0 < n0; r0 += 256) {
-      const int r = r0 + w;
-      float acc = 0.0f;
-      if (r > j && r < n0) {
-        const float* Wr = S + tri_ix(r, 0);
-        for (int m = j + 1 + part; m <= r; m += 4) acc = fmaf(Wr[m], S[tri_ix(m, j)], acc);
-      }
-      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-      acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-      if (part == 0 && r > j && r < n0) tr[r] = -d * acc;
-    }
-    __syncthreads();
-    for (int r = j + 1 + threadIdx.x; r < n0; r += blockDim.x) S[tri_ix(r, j)] = tr[r];
-    if (threadIdx.x == 0) S[tri_ix(j, j)] = d;
-    __syncthreads();
-  }
-  for (int e = threadIdx.x; e < n0 * n0; e += blockDim.x) {
-    const int r = e / n0, c = e - r * n0;
-    W[e] = c <= r ? S[tri_ix(r, c)] : 0.0f;
-  }
-  block_add_double(lsum, &chk->logdet);
-  if (threadIdx.x == 0) {
-    chk->bad = s_bad;
-    chk->min_piv = s_minpiv;
-  }
-}
-
-// Accepts the FP32 dense block or recomputes it in FP64.  The FP32 block's
-// error is estimated like a conditional's (rescue.cuh): every dense row is a
-// conditional on all earlier dense points, with K_jj = K_00 for every j, so
-// est = 2^-24 (K_00 / p_min)^2 from the smallest FP32 pivot p_min.  When the
-// estimate exceeds the kernel's rescue_tol or a pivot was floored, the block
-// is refactored from the coordinates in FP64 (K_00 from FP64 distances,
-// left-looking Cholesky with the same floor, inverse by forward substitution)
-// and rounded to FP32; else the FP32 block's log-determinant and floor count
-// are taken.  One block of 1024 threads; Lw, Ww are n0 x n0 FP64 work arrays.
-template <int KT>
-__global__ void __launch_bounds__(1024) dense_finish_kernel(
-    const float4* __restrict__ xs, int n0, KernF kf, const DenseCheck* __restrict__ chk,
-    double* __restrict__ Lw, double* __restrict__ Ww, float* __restrict__ L0,
-    float* __restrict__ L0inv, float* __restrict__ sigma, double* __restrict__ logdet,
-    unsigned long long* __restrict__ not_pd) {
-  extern __shared__ double tcol[];  // [n0]
-  __shared__ unsigned long long s_bad;
-  const float k0f = kf.s2 + kf.nug;
-  const float r32 = k0f / chk->min_piv;
-  const bool redo = chk->bad > 0 || !(r32 * r32 <= kf.resc_T);
-  if (!redo) {
-    if (threadIdx.x == 0) {
-      atomicAdd(logdet, chk->logdet);
-      if (chk->bad) atomicAdd(not_pd, chk->bad);
-    }
-    return;
-  }
-  if (threadIdx.x == 0) s_bad = 0;
-  const double k0 = kf.s2d + kf.nugd;
-  for (int64_t e = threadIdx.x; e < (int64_t)n0 * n0; e += blockDim.x) {
-    const int i = (int)(e / n0), j = (int)(e % n0);
-    Lw[e] = j < i ? kappa64<KT>(kf, dist64(xs[i], xs[j])) : (j == i ? k0 : 0.0);
-  }
-  __syncthreads();
-  const double fl = kPdFloor64 * k0;
-  for (int j = 0; j < n0; j++) {
-    const double* Lj = Lw + (int64_t)j * n0;
-    for (int r = j + threadIdx.x; r < n0; r += blockDim.x) {
-      const double* Lr = Lw + (int64_t)r * n0;
-      double t = Lr[j];
-      for (int m = 0; m < j; m++) t -= Lr[m] * Lj[m];
-      tcol[r] = t;
-    }
-    __syncthreads();
-    double piv = tcol[j];
-    if (!(piv > fl)) piv = fl;
-    const double ljj = sqrt(piv);
-    for (int r = j + 1 + threadIdx.x; r < n0; r += blockDim.x) Lw[(int64_t)r * n0 + j] = tcol[r] / ljj;
-    if (threadIdx.x == 0) {
-      Lw[(int64_t)j * n0 + j] = ljj;
-      if (!(tcol[j] > fl)) s_bad++;
-    }
-    __syncthreads();
-  }
-  // L^-1 column by column (forward substitution), one column per thread
-  for (int c = threadIdx.x; c < n0; c += blockDim.x) {
-    Ww[(int64_t)c * n0 + c] = 1.0 / Lw[(int64_t)c * n0 + c];
-    for (int i = c + 1; i < n0; i++) {
-      const double* Li = Lw + (int64_t)i * n0;
-      double t = 0.0;
-      for (int m = c; m < i; m++) t += Li[m] * Ww[(int64_t)m * n0 + c];
-      Ww[(int64_t)i * n0 + c] = -t / Li[i];
-    }
-  }
-  __syncthreads();
-  double lsum = 0.0;
-  for (int64_t e = threadIdx.x; e < (int64_t)n0 * n0; e += blockDim.x) {
-    const int i = (int)(e / n0), j = (int)(e % n0);
-    L0[e] = j <= i ? (float)Lw[e] : 0.0f;
-    L0inv[e] = j <= i ? (float)Ww[e] : 0.0f;
-    if (i == j) {
-      const float l = (float)Lw[e];
-      sigma[i] = l;
-      lsum += log((double)l * (double)l);
-    }
-  }
-  block_add_double(lsum, logdet);
-  if (threadIdx.x == 0 && s_bad) atomicAdd(not_pd, s_bad);
-}
-
 template <int G>
 int launch_point(int type, graphgp_graph_t g, graphgp_factor_t f, const KernF& kf,
                  const RescueList& rl, const RowView& rv, cudaStream_t s) {
@@ -702,49 +428,6 @@ int point_factor_rows(graphgp_graph_t g, graphgp_factor_t f, const KernF& kf, in
 int point_factor(graphgp_graph_t g, graphgp_factor_t f, const KernF& kf, int type,
                  cudaStream_t s) {
   return point_factor_rows(g, f, kf, type, 0, g->N - g->n0, s);
-}
-
-int dense_factor(graphgp_graph_t g, graphgp_factor_t f, const KernF& kf, int type,
-                 cudaStream_t s) {
-  int n0 = g->n0;
-  unsigned grid = grid_for((int64_t)n0 * n0, 256);
-  switch (type) {
-    case GRAPHGP_MATERN12: dense_fill_kernel<GRAPHGP_MATERN12><<<grid, 256, 0, s>>>(g->xs, n0, kf, f->L0); break;
-    case GRAPHGP_MATERN32: dense_fill_kernel<GRAPHGP_MATERN32><<<grid, 256, 0, s>>>(g->xs, n0, kf, f->L0); break;
-    case GRAPHGP_MATERN52: dense_fill_kernel<GRAPHGP_MATERN52><<<grid, 256, 0, s>>>(g->xs, n0, kf, f->L0); break;
-    default: dense_fill_kernel<GRAPHGP_SQEXP><<<grid, 256, 0, s>>>(g->xs, n0, kf, f->L0); break;
-  }
-  GGP_CUDA(cudaGetLastError());
-  Scratch sc(s);
-  DenseCheck* chk = nullptr;
-  double* work = nullptr;
-  GGP_TRY(sc.alloc(&chk, 1));
-  GGP_TRY(sc.alloc(&work, 2 * (size_t)n0 * n0));
-  GGP_CUDA(cudaMemsetAsync(chk, 0, sizeof(DenseCheck), s));
-  if (n0 <= kDenseSmemMax) {
-    const size_t smem = ((size_t)n0 * (n0 + 1) / 2 + n0) * sizeof(float);
-    GGP_CUDA(cudaFuncSetAttribute(dense_chol_smem_kernel,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dense_chol_smem_kernel<<<1, 1024, smem, s>>>(f->L0, f->L0inv, n0, f->sigma, chk);
-  } else {
-    dense_chol_kernel<<<1, 1024, n0 * sizeof(float), s>>>(f->L0, f->L0inv, n0, f->sigma, chk);
-  }
-  GGP_CUDA(cudaGetLastError());
-  double* Lw = work;
-  double* Ww = work + (size_t)n0 * n0;
-  const size_t smem64 = (size_t)n0 * sizeof(double);
-#define GGP_DF(KT)                                                                             \
-  dense_finish_kernel<KT><<<1, 1024, smem64, s>>>(g->xs, n0, kf, chk, Lw, Ww, f->L0, f->L0inv, \
-                                                  f->sigma, f->logdet, f->not_pd)
-  switch (type) {
-    case GRAPHGP_MATERN12: GGP_DF(GRAPHGP_MATERN12); break;
-    case GRAPHGP_MATERN32: GGP_DF(GRAPHGP_MATERN32); break;
-    case GRAPHGP_MATERN52: GGP_DF(GRAPHGP_MATERN52); break;
-    default: GGP_DF(GRAPHGP_SQEXP); break;
-  }
-#undef GGP_DF
-  GGP_CUDA(cudaGetLastError());
-  return GRAPHGP_OK;
 }
 
 }  // namespace ggp
