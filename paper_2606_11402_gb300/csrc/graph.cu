@@ -341,11 +341,17 @@ extern "C" int graphgp_build_graph(const float* points_d, int64_t N, int d, int 
     g->has_tree = true;
     int32_t* node_at_inorder = nullptr;
     GGP_TRY(sc.alloc(&node_at_inorder, N));
-    GGP_TRY(tree_build(g->pts_in, N, rule, g->tree_point, g->split_dim, g->inorder,
-                       node_at_inorder, s));
-    // preceding kNN
-    GGP_TRY(knn_query(g->pts_in, g->tree_point, g->split_dim, node_at_inorder, N, k, n0,
-                      g->nbr_tree, g->err, s));
+    int levels = 0;
+    while (((int64_t(1) << levels) - 1) < N) levels++;
+    {
+      Scratch bx(s);  // subtree boxes, only until the neighbours are found
+      float4* box = nullptr;
+      GGP_TRY(bx.alloc(&box, (size_t)2 << (levels - 1)));
+      GGP_TRY(tree_build(g->pts_in, N, rule, g->tree_point, g->split_dim, g->inorder,
+                         node_at_inorder, box, s));
+      // preceding kNN
+      GGP_TRY(knn_query(g->pts_in, g->tree_point, box, N, k, n0, g->nbr_tree, g->err, s));
+    }
     // depth
     GGP_CUDA(cudaMemsetAsync(g->depth_tree, 0, n0 * sizeof(int32_t), s));
     GGP_CUDA(cudaMemsetAsync(g->depth_tree + n0, 0xff, (N - n0) * sizeof(int32_t), s));

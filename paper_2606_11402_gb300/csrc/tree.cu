@@ -69,7 +69,8 @@ __global__ void level_nodes_kernel(const float* __restrict__ pts, int64_t N,
                                    int32_t* __restrict__ tree_point,
                                    uint8_t* __restrict__ split_dim,
                                    int32_t* __restrict__ inorder,
-                                   int32_t* __restrict__ node_at_inorder) {
+                                   int32_t* __restrict__ node_at_inorder,
+                                   float4* __restrict__ box) {
   int64_t first = (int64_t(1) << l) - 1;
   int64_t count = int64_t(1) << l;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < count;
@@ -81,14 +82,21 @@ __global__ void level_nodes_kernel(const float* __restrict__ pts, int64_t N,
     int64_t m = subtree_nodes(lc, N);
     int64_t st = start[j];
     int dim;
-    if (rule == 0) {
-      float ext[3];
+    float lo[3], hi[3], ext[3];
+    if (rule == 0 || box) {
 #pragma unroll
       for (int d = 0; d < 3; d++) {
-        float lo = pts[3 * (int64_t)ord.o[d][st] + d];
-        float hi = pts[3 * (int64_t)ord.o[d][st + S - 1] + d];
-        ext[d] = __fsub_rn(hi, lo);
+        lo[d] = pts[3 * (int64_t)ord.o[d][st] + d];
+        hi[d] = pts[3 * (int64_t)ord.o[d][st + S - 1] + d];
+        ext[d] = __fsub_rn(hi[d], lo[d]);
       }
+    }
+    if (box) {
+      const int64_t h = tree_heap_index(j);
+      box[2 * h] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+      box[2 * h + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
+    }
+    if (rule == 0) {
       dim = 0;
       if (ext[1] > ext[dim]) dim = 1;
       if (ext[2] > ext[dim]) dim = 2;
@@ -192,7 +200,7 @@ __global__ void part_scatter_kernel(int64_t N, int A,
 
 int tree_build(const float* pts, int64_t N, int rule, int32_t* tree_point,
                uint8_t* split_dim, int32_t* inorder, int32_t* node_at_inorder,
-               cudaStream_t s) {
+               float4* box, cudaStream_t s) {
   if (N <= 0) return GRAPHGP_OK;
   Scratch sc(s);
   int32_t* ord[3][2];
@@ -232,7 +240,8 @@ int tree_build(const float* pts, int64_t N, int rule, int32_t* tree_point,
     int64_t nodes = int64_t(1) << l;
     level_nodes_kernel<<<grid_for(nodes, B), B, 0, s>>>(pts, N, l, rule, o, start, msize,
                                                         tree_point, split_dim, inorder,
-                                                        node_at_inorder);
+                                                        node_at_inorder,
+                                                        l < levels - 1 ? box : nullptr);
     GGP_CUDA(cudaGetLastError());
     if (l == levels - 1) break;  // last level: every subtree is a single node
     slot_side_kernel<<<grid, B, 0, s>>>(N, o, seg[sg], seg[1 - sg], start, msize, split_dim,
