@@ -248,33 +248,43 @@ __global__ void __launch_bounds__(128) point_factor_wide_kernel(
 
 // The FP64 rows listed by the factor kernels: b (row stride kp), sigma, and
 // their log-determinant and floor counts.
-// k <= 32: one warp per listed row (warp_row_factor64, the routine of every
-// other rescue of these k).
+// k <= 32: several rows per warp (group_row_factor64).
+constexpr int kRescueWarps = 4;
+
 template <int KMAX, int KT>
-__global__ void __launch_bounds__(128) factor_rescue_warp_kernel(
+__global__ void __launch_bounds__(32 * kRescueWarps) factor_rescue_group_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int k, int kp, int64_t n0,
     KernF kf, RescueList rl, float* __restrict__ b_out, float* __restrict__ sigma_out,
     double* __restrict__ logdet, unsigned long long* __restrict__ not_pd) {
-  __shared__ double Wsm[4][KMAX * (KMAX + 1)];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  using GR = GroupRow64<KMAX>;
+  extern __shared__ __align__(16) unsigned char rsm[];
+  const int lane = threadIdx.x & 31, grp = threadIdx.x / GR::G, g = threadIdx.x % GR::G;
+  GR& R = reinterpret_cast<GR*>(rsm)[grp];
   LogAcc acc;
   unsigned long long clamped_rows = 0;
   const unsigned long long cnt = *rl.count;
   const int64_t n = (int64_t)(cnt < rl.cap ? cnt : rl.cap);
-  for (int64_t r = blockIdx.x * 4 + warp; r < n; r += (int64_t)gridDim.x * 4) {
-    const int64_t i = rl.rows[r];
-    const int64_t t = i - n0;
-    const WarpRow64 w = warp_row_factor64<KMAX, KT>(xs, nbr + t * kp, k, __ldg(xs + i), kf,
-                                                    Wsm[warp]);
-    if (lane < kp) b_out[t * kp + lane] = lane < k ? (float)w.b : 0.0f;
-    if (lane == 0) {
-      const float sg = (float)w.sigma;
-      sigma_out[i] = sg;
-      acc.mul(sg);
-      if (w.clamped) clamped_rows++;
+  constexpr int kPerBlock = kRescueWarps * GR::kRows;
+  const int64_t wrow = (threadIdx.x >> 5) * GR::kRows;  // the warp's first row in the block's
+  for (int64_t r0 = (int64_t)blockIdx.x * kPerBlock + wrow; r0 < n;
+       r0 += (int64_t)gridDim.x * kPerBlock) {  // the same on every lane
+    const int64_t r = r0 + lane / GR::G;
+    const bool act = r < n;
+    const int64_t i = act ? rl.rows[r] : n0, t = i - n0;
+    bool clamped;
+    const double sigma = group_row_factor64<KMAX, KT>(R, act, xs, nbr + t * kp, k, __ldg(xs + i), kf,
+                                                      clamped);
+    if (act) {
+      for (int a = g; a < kp; a += GR::G) b_out[t * kp + a] = a < k ? (float)R.y[a] : 0.0f;
+      if (g == 0) {
+        const float sg = (float)sigma;
+        sigma_out[i] = sg;
+        acc.mul(sg);
+        if (clamped) clamped_rows++;
+      }
     }
   }
-  block_add_double(lane == 0 ? acc.log_value() : 0.0, logdet);
+  block_add_double(acc.log_value(), logdet);
   for (int o = 16; o; o >>= 1) clamped_rows += __shfl_xor_sync(0xffffffffu, clamped_rows, o);
   if (lane == 0 && clamped_rows) atomicAdd(not_pd, clamped_rows);
 }
@@ -312,7 +322,9 @@ int launch_rescue(int type, graphgp_graph_t g, graphgp_factor_t f, const KernF& 
   const unsigned grid = 4 * (unsigned)num_sms();
 #define GGP_RS(KT)                                                                          \
   if constexpr (KMAX <= 32) {                                                               \
-    factor_rescue_warp_kernel<KMAX, KT><<<grid, 128, 0, s>>>(                               \
+    constexpr size_t smem = kRescueWarps * GroupRow64<KMAX>::kRows * sizeof(GroupRow64<KMAX>); \
+    GGP_CUDA(allow_dyn_smem(factor_rescue_group_kernel<KMAX, KT>, smem));                   \
+    factor_rescue_group_kernel<KMAX, KT><<<grid, 32 * kRescueWarps, smem, s>>>(             \
         g->xs, rv.nbr, g->k, g->kp, rv.n0, kf, rl, rv.b, f->sigma, f->logdet, f->not_pd);   \
   } else {                                                                                  \
     factor_rescue_kernel<KMAX, KT><<<grid, 128, 0, s>>>(                                    \

@@ -208,6 +208,102 @@ __device__ __noinline__ WarpRow64 warp_row_factor64(const float4* __restrict__ x
   return WarpRow64{real ? b : 0.0, sqrt(s2), clamped};
 }
 
+// The same conditional for a list of rows (k <= KMAX <= 32): G lanes per row,
+// 32 / G rows per warp, in the same operations on every entry, so the bits
+// agree with warp_row_factor64.  A warp instruction in FP64 takes 16 cycles
+// here however many of its lanes work, so what counts is the number of lanes
+// that do: one warp per row left three quarters of them idle in the kernel
+// values and the whole warp waiting for each pivot's root and quotients; eight
+// rows share those now, and a row's k (k + 1) / 2 values are dealt over its
+// lanes.  Lane g owns the rows a = g mod G of the matrix, in shared memory.
+template <int KMAX>
+struct GroupRow64 {
+  static constexpr int G = KMAX <= 16 ? 4 : 8;
+  static constexpr int kRows = 32 / G;  // per warp
+  double L[KMAX * (KMAX + 1) / 2 + 1];  // odd count: rows of a warp on different banks
+  double y[KMAX];
+  float4 x[KMAX];
+};
+
+// All 32 lanes call it; `act`: the group has a row.  b is left in R.y; returns
+// sigma and the floor flag.
+template <int KMAX, int KT>
+__device__ __forceinline__ double group_row_factor64(GroupRow64<KMAX>& R, bool act,
+                                                     const float4* __restrict__ xs,
+                                                     const int32_t* row, int k, float4 xq,
+                                                     const KernF& p, bool& clamped) {
+  constexpr int G = GroupRow64<KMAX>::G;
+  const int g = threadIdx.x % G;
+  const double k0 = kappa64<KT>(p, 0.0) + p.nugd;
+  const double fl = kPdFloor64 * k0;
+  __syncwarp();
+  if (act)
+    for (int a = g; a < k; a += G) R.x[a] = __ldg(xs + row[a]);
+  __syncwarp();
+  if (act) {
+    int a = 0, c = g;  // entry e = g, g + G, ... of the lower triangle, by rows
+    const int n = k * (k + 1) / 2;
+    for (int e = g; e < n; e += G) {
+      while (c > a) c -= ++a;
+      R.L[e] = c == a ? k0 : kappa64<KT>(p, dist64(R.x[a], R.x[c]));
+      c += G;
+    }
+    for (int b = g; b < k; b += G) R.y[b] = kappa64<KT>(p, dist64(R.x[b], xq));
+  }
+  __syncwarp();
+  clamped = false;
+  double s2 = k0;
+  for (int j = 0; j < k; j++) {
+    double ljj = 1.0, yj = 0.0;
+    if (act) {
+      double piv = R.L[tri64(j, j)];
+      if (!(piv > fl)) {
+        piv = fl;
+        clamped = true;
+      }
+      ljj = sqrt(piv);
+      yj = R.y[j] / ljj;
+      s2 -= yj * yj;
+    }
+    __syncwarp();  // every lane has read L_jj and y_j
+    if (act) {
+      if (j % G == g) {
+        R.L[tri64(j, j)] = ljj;
+        R.y[j] = yj;
+      }
+      for (int a = j + 1 + (g + 2 * G - (j + 1) % G) % G; a < k; a += G) {
+        const double laj = R.L[tri64(a, j)] / ljj;
+        R.L[tri64(a, j)] = laj;
+        R.y[a] -= laj * yj;
+      }
+    }
+    __syncwarp();
+    if (act)
+      for (int a = j + 1 + (g + 2 * G - (j + 1) % G) % G; a < k; a += G) {
+        double* La = R.L + tri64(a, 0);
+        const double laj = La[j];
+        for (int c = j + 1; c <= a; c++) La[c] -= laj * R.L[tri64(c, j)];
+      }
+    __syncwarp();
+  }
+  if (!(s2 > fl)) {
+    s2 = fl;
+    clamped = true;
+  }
+  // b = L^-T y, last entry first
+  for (int j = k - 1; j >= 0; j--) {
+    double bj = 0.0;
+    if (act) bj = R.y[j] / R.L[tri64(j, j)];
+    __syncwarp();
+    if (act) {
+      if (j % G == g) R.y[j] = bj;
+      for (int a = g; a < j; a += G) R.y[a] -= R.L[tri64(j, a)] * bj;
+    }
+    __syncwarp();
+  }
+  return sqrt(s2);
+}
+
 // The row's contribution to thetabar = (d/dl, d/dsigma2, d/dnugget) from the
 // cotangents of its weights, bbar_a = alpha v_c(a), and of its conditional
 // standard deviation, sigbar (Sec. 2.3; with s = sigma^2, g = K_cc^-1 bbar:
