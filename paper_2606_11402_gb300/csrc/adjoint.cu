@@ -23,7 +23,7 @@
 // theta = (lengthscale, sigma2, nugget); theta_bar is accumulated in FP64.
 #include <algorithm>
 
-#include "pointpair.cuh"
+#include "pointoct.cuh"
 #include "pointwide.cuh"
 
 namespace ggp {
@@ -250,111 +250,51 @@ int whiten_adjoint_scatter(graphgp_graph_t g, graphgp_factor_t f, const float* x
 }
 
 // ---- per-row factor backward ------------------------------------------------------
-// Lane a's row of Kbar against dK/dtheta for the G-lane group form, after
-// g = K_cc^-1 bbar (lane a holds g_a): Kbar_ac = -g_a b_c + sbar b_a b_c,
-// Kbar_ai = g_a - 2 sbar b_a, Kbar_ii = sbar (lane 0); the three partial
-// sums come back reduced over the group (every lane holds them).
-template <int G, int KT>
-__device__ __forceinline__ void group_row_theta(const PointState<G>& st, int a, int k, bool real,
-                                                const KernF& kf, float g, float sbar, float& pl,
-                                                float& ps, float& pn) {
-  const unsigned full = 0xffffffffu;
-  const float inv_s2 = 1.0f / kf.s2;
-  pl = ps = pn = 0.0f;
-  const float ba = st.b_own;
-#pragma unroll
-  for (int c = 0; c < G; c++) {
-    if (c >= k) break;
-    const float bc = __shfl_sync(full, st.b_own, c, G);
-    const float kb = -g * bc + sbar * ba * bc;
-    if (c == a) {
-      ps += kb;
-      pn += kb;
-    } else {
-      const KD kd = kappa_dkappa_d2<KT>(kf, st.D2[c]);
-      ps += kb * kd.k * inv_s2;
-      pl += kb * kd.dl;
-    }
-  }
-  {
-    const float kci = g - 2.0f * sbar * ba;
-    const KD kd = kappa_dkappa_d2<KT>(kf, st.d2q);
-    ps += kci * kd.k * inv_s2;
-    pl += kci * kd.dl;
-  }
-  if (!real) pl = ps = pn = 0.0f;
-  if (a == 0) {  // Kbar_ii = sbar
-    ps += sbar;
-    pn += sbar;
-  }
-#pragma unroll
-  for (int o = G / 2; o; o >>= 1) {
-    pl += __shfl_xor_sync(full, pl, o, G);
-    ps += __shfl_xor_sync(full, ps, o, G);
-    pn += __shfl_xor_sync(full, pn, o, G);
-  }
-}
-
 // mode 0 (whiten): alpha_i = -xibar_i / sigma_i, beta = 2 logdetbar.
 // mode 1 (generate): alpha_i = u_i, beta = 0; also writes xibar_i = sigma_i u_i.
 // bbar_i = alpha_i v_c(i), sigbar_i = alpha_i xi_i + beta / sigma_i.
-template <int G, int KT>
-__global__ void __launch_bounds__(128) factor_backward_kernel(
+// 16 < k <= 32: eight lanes per point, the factor recomputed by oct_factor
+// (bit-identical b and sigma to the forward kernel).  Rows the forward factor
+// recomputed in FP64 (rescue.cuh) go to factor_backward_rescue_kernel, whose
+// list holds every row.
+template <int K, int KT>
+__global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) factor_backward_oct_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int kp,
     int64_t n0, KernF kf, int mode, const float* __restrict__ coef, float beta,
     const float* __restrict__ v, const float* __restrict__ xi, float* __restrict__ xibar_out,
     double* __restrict__ thetabar, int64_t* __restrict__ rescue_rows,
     unsigned long long* __restrict__ rescue_count) {
-  constexpr int PPW = 32 / G;
-  constexpr int GS = PFLayout<G>::GS;
-  __shared__ __align__(16) float Ls[4 * PPW * GS];
-  const int lane = threadIdx.x & 31;
-  const int grp = lane / G;
-  const int a = lane % G;
-  const int warp = threadIdx.x >> 5;
-  const unsigned full = 0xffffffffu;
-  float* Lg = Ls + (warp * PPW + grp) * GS;
+  using OL = OctLayout<K>;
+  extern __shared__ __align__(16) float psm[];
+  const int lane = threadIdx.x & 31, r = lane & 7, first = (threadIdx.x >> 5) * 4;
+  float* S = psm + (threadIdx.x >> 3) * OL::kStride;
+  const uint64_t pol_v = l2_evict_last();
   double tl = 0.0, ts = 0.0, tn = 0.0;
-  const int64_t total_groups = (int64_t)gridDim.x * 4 * PPW;
-  const int64_t gid = ((int64_t)blockIdx.x * 4 + warp) * PPW + grp;
   const int64_t npts = N - n0;
-  const int64_t iters = (npts + total_groups - 1) / total_groups;
-  for (int64_t it = 0; it < iters; it++) {
-    int64_t t = it * total_groups + gid;
-    bool valid = t < npts;
-    int64_t i = n0 + (valid ? t : 0);
-    bool real = a < k;
-    int32_t ca = real ? nbr[(i - n0) * kp + a] : 0;
-    PointState<G> st;
-    point_factor_group<G, KT>(st, a, k, kf, xs[ca], xs[i], Lg);
-    __syncwarp();
-    float sigma = st.sigma;
-    float ci = coef[i];
-    float alpha = mode == 0 ? -ci / sigma : ci;
-    float xii = xi[i];
-    float sigbar = alpha * xii + beta / sigma;
-    float sbar = sigbar / (2.0f * sigma);
-    float bbar = real ? alpha * v[ca] : 0.0f;
-    float g = group_chol_solve<G>(st, a, k, bbar, Lg);
-    __syncwarp();
-    // row a of Kbar against dK/dtheta
-    float pl, ps, pn;
-    group_row_theta<G, KT>(st, a, k, real, kf, g, sbar, pl, ps, pn);
-    // rows the forward factor recomputed in FP64 (rescue.cuh): the FP32 sums
-    // above are discarded and the row goes to factor_backward_rescue_kernel
-    const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (grp * G));
-    const bool lane_bad = real && !isfinite(st.b_own);
-    const bool rescue = st.clamped || row_error_too_large(st.max_ratio, st.varw, st.sigma, kf) ||
-                        !isfinite(st.sigma) || (__ballot_sync(full, lane_bad) & gmask);
-    if (valid && a == 0) {
-      if (rescue) {
+  const int64_t stride = (int64_t)gridDim.x * OL::kPoints;
+  for (int64_t b0 = (int64_t)blockIdx.x * OL::kPoints; b0 < npts; b0 += stride) {
+    __syncthreads();  // the warps of a block share the instruction stream
+    const int64_t t = b0 + first + (lane >> 3);
+    const bool valid = t < npts;
+    const int64_t tt = valid ? t : npts - 1, i = n0 + tt;
+    const int32_t* row = nbr + tt * kp;
+    const float4 xq = __ldg(xs + i);
+    oct_stage<K>(S, r, xs, row, kp);
+    OctFactor<K> f;
+    oct_factor<K, KT>(f, S, r, k, kf, xq);
+    const bool rescue = valid && oct_needs_rescue(f, kf);
+    const float ci = coef[i], xii = xi[i];
+    const float alpha = mode == 0 ? -ci / f.sigma : ci;
+    const float sigbar = alpha * xii + beta / f.sigma;
+    float vv[K / 8];
+    oct_gather<K, false>(vv, r, k, row, v, pol_v);
+    oct_row_backward<K, KT>(f, S, r, k, kf, xq, vv, alpha, sigbar / (2.0f * f.sigma),
+                            valid && !rescue, tl, ts, tn);
+    if (valid && r == 0) {
+      if (rescue)
         rescue_rows[atomicAdd(rescue_count, 1ull)] = i;
-      } else {
-        tl += pl;
-        ts += ps;
-        tn += pn;
-        if (mode == 1) xibar_out[i] = sigma * ci;
-      }
+      else if (mode == 1)
+        xibar_out[i] = f.sigma * ci;
     }
   }
   block_add3(tl, ts, tn, thetabar);
@@ -473,8 +413,7 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) factor_b
   const int lane = threadIdx.x & 31, r = lane & 1, first = (threadIdx.x >> 5) * 16;
   float* S = psm + (threadIdx.x >> 1) * PL::kStride;
   const uint64_t pol_v = l2_evict_last();
-  double tl = 0.0, ts = 0.0, tn = 0.0;   // scaled sums of the FP32 rows
-  double wl = 0.0, ws = 0.0, wn = 0.0;   // rows recomputed here in FP64
+  double tl = 0.0, ts = 0.0, tn = 0.0;
   const int64_t npts = N - n0;
   const int64_t stride = (int64_t)gridDim.x * PL::kPoints;
   PairLoad<K> ld;
@@ -510,13 +449,13 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) factor_b
         const float sg = (float)R.sigma;
         const double al = mode == 0 ? -(double)ci / sg : (double)ci;
         const double sb = al * (double)xii + (double)beta / sg;
-        row_backward64<K, KT>(R, xs, row_ptr, k, xq, kf, v, al, sb, sg, wl, ws, wn);
+        row_backward64<K, KT>(R, xs, row_ptr, k, xq, kf, v, al, sb, sg, tl, ts, tn);
         if (mode == 1) xibar_out[i] = sg * ci;
       }
     }
     __syncwarp();
   }
-  block_add3(wl + tl * theta_scale<KT>(kf), ws + ts, wn + tn, thetabar);
+  block_add3(tl, ts, tn, thetabar);
 }
 
 // NLL value and gradient in one pass, the factors recomputed and never stored
@@ -545,7 +484,7 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) nll_grad
   float* S = psm + (threadIdx.x >> 1) * PL::kStride;
   const uint64_t pol_v = l2_evict_last();
   LogAcc lacc;
-  double sq = 0.0, tl = 0.0, ts = 0.0, tn = 0.0, wl = 0.0, ws = 0.0, wn = 0.0;
+  double sq = 0.0, tl = 0.0, ts = 0.0, tn = 0.0;
   unsigned long long clamped = 0;
   const int64_t npts = N - n0;
   const int64_t stride = (int64_t)gridDim.x * PL::kPoints;
@@ -618,13 +557,13 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) nll_grad
           const float s64 = (float)R.sigma;
           const double al = -(double)xbu / s64;
           const double sb = al * (double)xu0 + (double)nllbar / s64;
-          row_backward64<K, KT>(R, xs, row, k, xu, kf, v, al, sb, s64, wl, ws, wn);
+          row_backward64<K, KT>(R, xs, row, k, xu, kf, v, al, sb, s64, tl, ts, tn);
         }
       }
     }
     __syncwarp();
   }
-  block_add3(wl + tl * theta_scale<KT>(kf), ws + ts, wn + tn, thetabar);
+  block_add3(tl, ts, tn, thetabar);
   block_add_double(sq, acc);
   block_add_double(lacc.log_value(), acc + 1);
   unsigned long long c = clamped;
@@ -632,105 +571,91 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) nll_grad
   if (lane == 0 && c) atomicAdd(not_pd, c);
 }
 
-// The FP64 conditional of a warp's row out of line: the rescue is rare, and
-// inlined its state would raise the register count of the whole kernel.
-template <int KT>
-__device__ __noinline__ WarpRow64 warp_row_factor64_outlined(const float4* __restrict__ xs,
-                                                            const int32_t* row, int k,
-                                                            float4 xq, KernF kf, double* W) {
-  return warp_row_factor64<32, KT>(xs, row, k, xq, kf, W);
-}
-
-// The one-pass NLL value and gradient for 16 < k <= 32: one warp per point,
-// the 32-lane group factor (point_factor_group with the factor kernel's
-// rescue decision), so b and sigma are the stored factor's; a row that needs
-// FP64 takes its b and sigma from warp_row_factor64 for the value and the
-// scatter and is listed for factor_backward_rescue_kernel (the list holds
-// every row); the other rows run the group backward (group_chol_solve,
-// group_row_theta) on the factor still in the warp's shared memory.
-template <int KP, int KT>
-__global__ void __launch_bounds__(128, 3) nll_grad_fused_group_kernel(
+// The one-pass NLL value and gradient for 16 < k <= 32: eight lanes per point,
+// as nll_grad_fused_kernel with the factor of pointoct.cuh.  Rows that need
+// FP64 follow the others of their warp and are listed for
+// factor_backward_rescue_kernel (the list holds every row).
+template <int K, int KP, int KT>
+__global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) nll_grad_fused_oct_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int64_t n0,
     KernF kf, float nllbar, const float* __restrict__ v, float* vbar, float* __restrict__ xi_out,
     float* __restrict__ xibar_out, double* __restrict__ thetabar, double* __restrict__ acc,
     unsigned long long* __restrict__ not_pd, int64_t* __restrict__ rescue_rows,
     unsigned long long* __restrict__ rescue_count) {
-  constexpr int GS = PFLayout<32>::GS;
-  __shared__ __align__(16) float Ls[4 * GS];
-  extern __shared__ __align__(16) double gws[];  // 4 x 32 x 33 doubles (FP64 rescue)
-  const int a = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  using OL = OctLayout<K>;
+  extern __shared__ __align__(16) float psm[];
   const unsigned full = 0xffffffffu;
-  float* Lg = Ls + warp * GS;
-  double* W = gws + warp * (32 * 33);
+  const int lane = threadIdx.x & 31, r = lane & 7, first = (threadIdx.x >> 5) * 4;
+  float* S = psm + (threadIdx.x >> 3) * OL::kStride;
   const uint64_t pol_v = l2_evict_last();
   LogAcc lacc;
   double sq = 0.0, tl = 0.0, ts = 0.0, tn = 0.0;
   unsigned long long clamped = 0;
   const int64_t npts = N - n0;
-  const int64_t nw = (int64_t)gridDim.x * 4;
-  for (int64_t t = (int64_t)blockIdx.x * 4 + warp; t < npts; t += nw) {  // warp-uniform
-    const int64_t i = n0 + t;
-    const int32_t* row = nbr + t * KP;
-    const bool real = a < k;
-    const int32_t ca = real ? __ldg(row + a) : 0;
+  const int64_t stride = (int64_t)gridDim.x * OL::kPoints;
+  for (int64_t b0 = (int64_t)blockIdx.x * OL::kPoints; b0 < npts; b0 += stride) {
+    __syncthreads();  // the warps of a block share the instruction stream
+    const int64_t t = b0 + first + (lane >> 3);
+    const bool valid = t < npts;
+    const int64_t tt = valid ? t : npts - 1, i = n0 + tt;
+    const int32_t* row = nbr + tt * KP;
     const float4 xq = __ldg(xs + i);
-    PointState<32> st;
-    point_factor_group<32, KT>(st, a, k, kf, __ldg(xs + ca), xq, Lg);
-    __syncwarp();
-    const bool lane_bad = real && !isfinite(st.b_own);
-    const bool rescue = st.clamped || row_error_too_large(st.max_ratio, st.varw, st.sigma, kf) ||
-                        !isfinite(st.sigma) || __ballot_sync(full, lane_bad);
-    float b = real ? st.b_own : 0.0f, sigma = st.sigma;
-    bool clamp = st.clamped;
-    if (rescue) {
-      const WarpRow64 w = warp_row_factor64_outlined<KT>(xs, row, k, xq, kf, W);
-      b = real ? (float)w.b : 0.0f;
-      sigma = (float)w.sigma;
-      clamp = w.clamped;
-    }
-    const float dot = warp_dot_stored_order<KP, false>(b, row, v, pol_v);
-    float xv = 0.0f;
-    if (a == 0) xv = (ld_keep_f(v + i, pol_v) - dot) / sigma;
-    xv = __shfl_sync(full, xv, 0);
+    oct_stage<K>(S, r, xs, row, KP);
+    OctFactor<K> f;
+    oct_factor<K, KT>(f, S, r, k, kf, xq);
+    const bool rescue = valid && oct_needs_rescue(f, kf), act = valid && !rescue;
+    float vv[K / 8];
+    oct_gather<K, false>(vv, r, k, row, v, pol_v);
+    const float sigma = f.sigma;
+    const float xv = (ld_keep_f(v + i, pol_v) - oct_dot<K>(f.b, vv, S, r, KP)) / sigma;
     const float xb = nllbar * xv;
     const float w = xb / sigma;
-    if (a == 0) {
-      sq += (double)xv * (double)xv;
-      lacc.mul(sigma);
-      clamped += clamp ? 1 : 0;
-      atomicAdd(vbar + i, w);
-    }
-    if (real && b != 0.0f) atomicAdd(vbar + ca, b * -w);
-    if (rescue) {
-      if (a == 0) {
-        xi_out[i] = xv;
-        xibar_out[i] = xb;
-        rescue_rows[atomicAdd(rescue_count, 1ull)] = i;
+    if (act) {
+      if (r == 0) {
+        sq += (double)xv * (double)xv;
+        lacc.mul(sigma);
+        clamped += f.clamped ? 1 : 0;
+        atomicAdd(vbar + i, w);
       }
-      __syncwarp();
-      continue;
+#pragma unroll
+      for (int s = 0; s < K / 8; s++)
+        if (8 * s + r < k && f.b[s] != 0.0f) atomicAdd(vbar + __ldg(row + 8 * s + r), f.b[s] * -w);
     }
     const float alpha = -xb / sigma;
     const float sigbar = alpha * xv + nllbar / sigma;
-    const float sbar = sigbar / (2.0f * sigma);
-    const float bbar = real ? alpha * v[ca] : 0.0f;
-    const float g = group_chol_solve<32>(st, a, k, bbar, Lg);
-    __syncwarp();
-    float pl, ps, pn;
-    group_row_theta<32, KT>(st, a, k, real, kf, g, sbar, pl, ps, pn);
-    if (a == 0) {
-      tl += pl;
-      ts += ps;
-      tn += pn;
+    oct_row_backward<K, KT>(f, S, r, k, kf, xq, vv, alpha, sigbar / (2.0f * sigma), act, tl, ts, tn);
+    unsigned m = __ballot_sync(full, rescue) & 0x01010101u;
+    while (m) {
+      const int src = __ffs(m) - 1;
+      m &= m - 1;
+      __syncwarp();
+      const int64_t u = b0 + first + (src >> 3), iu = n0 + u;
+      const int32_t* ru = nbr + u * KP;
+      const WarpRow64 wr = oct_row64<K, KT>(xs, ru, k, __ldg(xs + iu), kf,
+                                         reinterpret_cast<double*>(psm + first * OL::kStride));
+      const float b = lane < k ? (float)wr.b : 0.0f, sg = (float)wr.sigma;
+      const float dot = warp_dot_stored_order<KP, false>(b, ru, v, pol_v);
+      const float xu = __shfl_sync(full, (ld_keep_f(v + iu, pol_v) - dot) / sg, 0);
+      const float xbu = nllbar * xu, wu = xbu / sg;
+      if (lane < k && b != 0.0f) atomicAdd(vbar + ru[lane], b * -wu);
+      if (lane == src) {
+        sq += (double)xu * (double)xu;
+        lacc.mul(sg);
+        clamped += wr.clamped ? 1 : 0;
+        atomicAdd(vbar + iu, wu);
+        xi_out[iu] = xu;
+        xibar_out[iu] = xbu;
+        rescue_rows[atomicAdd(rescue_count, 1ull)] = iu;
+      }
     }
     __syncwarp();
   }
   block_add3(tl, ts, tn, thetabar);
   block_add_double(sq, acc);
-  block_add_double(a == 0 ? lacc.log_value() : 0.0, acc + 1);
+  block_add_double(lacc.log_value(), acc + 1);
   unsigned long long c = clamped;
   for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(full, c, o);
-  if (a == 0 && c) atomicAdd(not_pd, c);
+  if (lane == 0 && c) atomicAdd(not_pd, c);
 }
 
 __global__ void scale_kernel(const float* __restrict__ x, float s, float* __restrict__ y,
@@ -747,15 +672,15 @@ __global__ void mul_kernel(const float* __restrict__ a, const float* __restrict_
     y[i] = a[i] * x[i];
 }
 
-template <int G>
-int launch_factor_backward(graphgp_graph_t g, graphgp_factor_t f, int mode, const float* coef,
-                           float beta, const float* v, const float* xi, float* xibar,
-                           double* thetabar, const int32_t* nbr, int64_t N, int64_t n0v,
-                           cudaStream_t s) {
+template <int K>
+int launch_factor_backward_oct(graphgp_graph_t g, graphgp_factor_t f, int mode,
+                               const float* coef, float beta, const float* v, const float* xi,
+                               float* xibar, double* thetabar, const int32_t* nbr, int64_t N,
+                               int64_t n0v, cudaStream_t s) {
   int64_t npts = N - n0v;
   if (npts <= 0) return GRAPHGP_OK;
-  constexpr int PPW = 32 / G;
-  unsigned grid = grid_for((npts + 4 * PPW - 1) / (4 * PPW) * 128, 128, 16);
+  const unsigned grid = oct_grid<K>(npts);
+  constexpr size_t smem = OctLayout<K>::kBytes;
   KernF kf = make_kernf(f->kern);
   Scratch sc(s);
   int64_t* rows = nullptr;
@@ -765,10 +690,10 @@ int launch_factor_backward(graphgp_graph_t g, graphgp_factor_t f, int mode, cons
   GGP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
   const unsigned rgrid = (unsigned)num_sms() * 2;
 #define GGP_FB(KT)                                                                          \
-  factor_backward_kernel<G, KT><<<grid, 128, 0, s>>>(g->xs, nbr, N, g->k, g->kp, n0v, \
-                                                     kf, mode, coef, beta, v, xi, xibar,     \
-                                                     thetabar, rows, cnt);                   \
-  factor_backward_rescue_kernel<G, KT><<<rgrid, 128, 0, s>>>(                               \
+  GGP_CUDA(allow_dyn_smem(factor_backward_oct_kernel<K, KT>, smem));                        \
+  factor_backward_oct_kernel<K, KT><<<grid, kPairThreads, smem, s>>>(                       \
+      g->xs, nbr, N, g->k, g->kp, n0v, kf, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt); \
+  factor_backward_rescue_kernel<K, KT><<<rgrid, 128, 0, s>>>(                               \
       g->xs, nbr, g->k, g->kp, n0v, kf, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt, \
       (unsigned long long)npts)
   switch (f->kern.type) {
@@ -858,13 +783,14 @@ int launch_nll_grad_fused(graphgp_graph_t g, const graphgp_kernel* kern, float n
 }
 
 template <int KP>
-int launch_nll_grad_fused_group(graphgp_graph_t g, const graphgp_kernel* kern, float nllbar,
+int launch_nll_grad_fused_oct(graphgp_graph_t g, const graphgp_kernel* kern, float nllbar,
                                 const float* v, float* vbar, float* xi_tmp, float* xibar_tmp,
                                 double* thetabar, double* acc, unsigned long long* not_pd,
                                 cudaStream_t s) {
   const int64_t npts = g->N - g->n0;
   if (npts <= 0) return GRAPHGP_OK;
-  const unsigned grid = grid_for((npts + 3) / 4 * 128, 128, 16);
+  constexpr int K = KP <= 24 ? 24 : 32;
+  const unsigned grid = oct_grid<K>(npts);
   const KernF kf = make_kernf(*kern);
   Scratch sc(s);
   int64_t* rows = nullptr;
@@ -873,14 +799,13 @@ int launch_nll_grad_fused_group(graphgp_graph_t g, const graphgp_kernel* kern, f
   GGP_TRY(sc.alloc(&cnt, 1));
   GGP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
   const unsigned rgrid = (unsigned)num_sms() * 2;
-  constexpr size_t smem = (size_t)4 * 32 * 33 * sizeof(double);
+  constexpr size_t smem = OctLayout<K>::kBytes;
 #define GGP_NGG(KT)                                                                              \
-  GGP_CUDA(cudaFuncSetAttribute(nll_grad_fused_group_kernel<KP, KT>,                            \
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));        \
-  nll_grad_fused_group_kernel<KP, KT><<<grid, 128, smem, s>>>(                                   \
+  GGP_CUDA(allow_dyn_smem(nll_grad_fused_oct_kernel<K, KP, KT>, smem));                          \
+  nll_grad_fused_oct_kernel<K, KP, KT><<<grid, kPairThreads, smem, s>>>(                         \
       g->xs, g->nbr, g->N, g->k, g->n0, kf, nllbar, v, vbar, xi_tmp, xibar_tmp, thetabar, acc,  \
       not_pd, rows, cnt);                                                                        \
-  factor_backward_rescue_kernel<32, KT><<<rgrid, 128, 0, s>>>(                                   \
+  factor_backward_rescue_kernel<K, KT><<<rgrid, 128, 0, s>>>(                                   \
       g->xs, g->nbr, g->k, g->kp, g->n0, kf, 0, xibar_tmp, nllbar, v, xi_tmp, nullptr, thetabar, \
       rows, cnt, (unsigned long long)npts)
   switch (kern->type) {
@@ -947,9 +872,9 @@ int factor_backward_rows(graphgp_graph_t g, graphgp_factor_t f, int mode, const 
     case 12: return launch_factor_backward_pair<12>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
     case 16: return launch_factor_backward_pair<16>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
     case 20:
-    case 24:
+    case 24: return launch_factor_backward_oct<24>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
     case 28:
-    case 32: return launch_factor_backward<32>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
+    case 32: return launch_factor_backward_oct<32>(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
     default: return launch_factor_backward_wide(g, f, mode, coef, beta, v, xi, xibar, thetabar, nb, N, n0v, s);
   }
 }
@@ -1264,10 +1189,10 @@ extern "C" int graphgp_nll_grad_fused(graphgp_graph_t g, const graphgp_kernel* k
       case 8: rc = launch_nll_grad_fused<8>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
       case 12: rc = launch_nll_grad_fused<12>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
       case 16: rc = launch_nll_grad_fused<16>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
-      case 20: rc = launch_nll_grad_fused_group<20>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
-      case 24: rc = launch_nll_grad_fused_group<24>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
-      case 28: rc = launch_nll_grad_fused_group<28>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
-      default: rc = launch_nll_grad_fused_group<32>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
+      case 20: rc = launch_nll_grad_fused_oct<20>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
+      case 24: rc = launch_nll_grad_fused_oct<24>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
+      case 28: rc = launch_nll_grad_fused_oct<28>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
+      default: rc = launch_nll_grad_fused_oct<32>(g, kern, (float)nllbar, v_d, vbar_d, xi, xb, thetabar_d, acc, bad, s); break;
     }
     GGP_TRY(rc);
   }

@@ -2,19 +2,12 @@
 // block is in dense.cu.
 //
 // Per point i with c = c(i): b_i = K_ic K_cc^-1 and sigma_i^2 =
-// K_ii - K_ic K_cc^-1 K_ci.  A group of G lanes (G = 8, 16 or 32 >= k) of one
-// warp owns one point; lane a holds row a of K_cc in registers.  The
-// Cholesky factor is built column by column (left-looking): at step j every
-// lane forms its Schur value from its own row and row j of L, which lane j
-// published to shared memory in earlier steps; lane j's value is the pivot.
-// The forward solve y = L^-1 K_ci rides along (right-looking on the lanes'
-// K_ci entries), sigma^2 = K_ii - y.y is accumulated in compensated FP32
-// (two-sum / two-product), and b = L^-T y is a backward sweep reading L's
-// columns from shared memory.  Pivots below 1e-7 of their diagonal entry are
-// raised to that floor and counted.  logdet = sum log sigma_i^2 is reduced in
-// FP64 from the stored FP32 sigma (a running FP64 product with separate
-// exponent, one log per thread).
-#include "pointpair.cuh"
+// K_ii - K_ic K_cc^-1 K_ci, two lanes per point for k <= 16 (pointpair.cuh),
+// eight for k <= 32 (pointoct.cuh), a warp above (pointwide.cuh).  Pivots below
+// 1e-7 of their diagonal entry are raised to that floor and counted.  logdet =
+// sum log sigma_i^2 is reduced in FP64 from the stored FP32 sigma (a running
+// FP64 product with separate exponent, one log per thread).
+#include "pointoct.cuh"
 #include "pointwide.cuh"
 
 namespace ggp {
@@ -47,70 +40,49 @@ struct RowView {
   int64_t N, n0;
 };
 
-template <int G, int KT>
-__global__ void __launch_bounds__(128) point_factor_kernel(
+// 16 < k <= 32: eight lanes per point (pointoct.cuh), K = 24 or 32.
+template <int K, int KT>
+__global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) point_factor_oct_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int kp,
     int64_t n0, KernF kf, float* __restrict__ b_out, float* __restrict__ sigma_out,
     double* __restrict__ logdet, unsigned long long* __restrict__ not_pd, RescueList rl) {
-  constexpr int PPW = 32 / G;  // points per warp
-  constexpr int GS = PFLayout<G>::GS;
-  __shared__ __align__(16) float Ls[4 * PPW * GS];
-  // FP64 rescue workspace of each warp (dynamic: 4 G (G + 1) doubles)
-  extern __shared__ __align__(16) double gwsm[];
-  double* Wwarp = gwsm + (threadIdx.x >> 5) * (G * (G + 1));
-  const int lane = threadIdx.x & 31;
-  const int grp = lane / G;
-  const int a = lane % G;
-  const int warp = threadIdx.x >> 5;
-  float* Lg = Ls + (warp * PPW + grp) * GS;
+  using OL = OctLayout<K>;
+  extern __shared__ __align__(16) float psm[];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, r = lane & 7, first = (threadIdx.x >> 5) * 4;
+  float* S = psm + (threadIdx.x >> 3) * OL::kStride;
   LogAcc acc;
   unsigned long long clamped_rows = 0;
-  const int64_t total_groups = (int64_t)gridDim.x * 4 * PPW;
-  const int64_t gid = ((int64_t)blockIdx.x * 4 + warp) * PPW + grp;
   const int64_t npts = N - n0;
-  const int64_t iters = (npts + total_groups - 1) / total_groups;
-  for (int64_t it = 0; it < iters; it++) {
-    int64_t t = it * total_groups + gid;
-    bool valid = t < npts;
-    int64_t i = n0 + (valid ? t : 0);
-    int32_t ca = a < k ? nbr[(i - n0) * kp + a] : 0;
-    PointState<G> st;
-    point_factor_group<G, KT>(st, a, k, kf, xs[ca], xs[i], Lg);
-    __syncwarp();
-    // rescue decision, uniform over the group's lanes
-    const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (grp * G));
-    const bool lane_bad = a < k && !isfinite(st.b_own);
-    const bool rescue = st.clamped || row_error_too_large(st.max_ratio, st.varw, st.sigma, kf) ||
-                        !isfinite(st.sigma) || (__ballot_sync(0xffffffffu, lane_bad) & gmask);
-    static_assert(G == 32, "the group factor kernel runs one point per warp");
+  const int64_t stride = (int64_t)gridDim.x * OL::kPoints;
+  for (int64_t b0 = (int64_t)blockIdx.x * OL::kPoints; b0 < npts; b0 += stride) {
+    __syncthreads();  // the warps of a block share the instruction stream
+    const int64_t t = b0 + first + (lane >> 3);
+    const bool valid = t < npts;
+    const int64_t tt = valid ? t : npts - 1, i = n0 + tt;
+    const int32_t* row = nbr + tt * kp;
+    const float4 xq = __ldg(xs + i);
+    oct_stage<K>(S, r, xs, row, kp);
+    OctFactor<K> f;
+    oct_factor<K, KT>(f, S, r, k, kf, xq);
+    const bool rescue = valid && oct_needs_rescue(f, kf);
     bool deferred = false;
-    if (valid && rescue && a == 0) deferred = rl.defer(i);
-    deferred = __shfl_sync(0xffffffffu, deferred, 0);
-    if (valid && rescue && !deferred) {  // list full: the warp recomputes the row in place
-      const WarpRow64 w = warp_row_factor64<G, KT>(xs, nbr + (i - n0) * kp, k, xs[i], kf, Wwarp);
-      if (a < kp) b_out[(i - n0) * kp + a] = a < k ? (float)w.b : 0.0f;
-      if (a == 0) {
-        const float sg = (float)w.sigma;
-        sigma_out[i] = sg;
-        acc.mul(sg);
-        if (w.clamped) clamped_rows++;
-      }
-    }
-    if (valid && !deferred) {
-      if (rescue) {
-      } else {
-        if (a < kp) b_out[(i - n0) * kp + a] = a < k ? st.b_own : 0.0f;
-        if (a == 0) {
-          sigma_out[i] = st.sigma;
-          acc.mul(st.sigma);
-          if (st.clamped) clamped_rows++;
-        }
+    if (rescue && r == 0) deferred = rl.defer(i);
+    deferred = __shfl_sync(full, deferred, 0, 8);
+    oct_rescue<K, KT>(f, rescue && !deferred, psm + first * OL::kStride, r, xs, row, k, xq, kf);
+    if (valid && !deferred) {  // (a row that found the list full is recomputed by now)
+#pragma unroll
+      for (int s = 0; s < K / 8; s++)
+        if (8 * s + r < kp) b_out[tt * kp + 8 * s + r] = 8 * s + r < k ? f.b[s] : 0.0f;
+      if (r == 0) {
+        sigma_out[i] = f.sigma;
+        acc.mul(f.sigma);
+        if (f.clamped) clamped_rows++;
       }
     }
   }
-  double lv = (a == 0) ? acc.log_value() : 0.0;
-  block_add_double(lv, logdet);
-  for (int o = 16; o; o >>= 1) clamped_rows += __shfl_xor_sync(0xffffffffu, clamped_rows, o);
+  block_add_double(acc.log_value(), logdet);
+  for (int o = 16; o; o >>= 1) clamped_rows += __shfl_xor_sync(full, clamped_rows, o);
   if (lane == 0 && clamped_rows) atomicAdd(not_pd, clamped_rows);
 }
 
@@ -341,20 +313,15 @@ int launch_rescue(int type, graphgp_graph_t g, graphgp_factor_t f, const KernF& 
   return GRAPHGP_OK;
 }
 
-template <int G>
-int launch_point(int type, graphgp_graph_t g, graphgp_factor_t f, const KernF& kf,
-                 const RescueList& rl, const RowView& rv, cudaStream_t s) {
-  int64_t npts = rv.N - rv.n0;
-  constexpr int PPW = 32 / G;
-  int64_t groups_per_block = 4 * PPW;
-  unsigned grid = grid_for((npts + groups_per_block - 1) / groups_per_block * 128, 128, 16);
-  constexpr size_t smem = 4 * (size_t)G * (G + 1) * sizeof(double);
-#define GGP_PF(KT)                                                                       \
-  GGP_CUDA(cudaFuncSetAttribute(point_factor_kernel<G, KT>,                              \
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-  point_factor_kernel<G, KT><<<grid, 128, smem, s>>>(g->xs, rv.nbr, rv.N, g->k, g->kp,     \
-                                                     rv.n0, kf, rv.b, f->sigma, f->logdet, \
-                                                     f->not_pd, rl)
+template <int K>
+int launch_point_oct(int type, graphgp_graph_t g, graphgp_factor_t f, const KernF& kf,
+                     const RescueList& rl, const RowView& rv, cudaStream_t s) {
+  const unsigned grid = oct_grid<K>(rv.N - rv.n0);
+  constexpr size_t smem = OctLayout<K>::kBytes;
+#define GGP_PF(KT)                                                                             \
+  GGP_CUDA(allow_dyn_smem(point_factor_oct_kernel<K, KT>, smem));                              \
+  point_factor_oct_kernel<K, KT><<<grid, kPairThreads, smem, s>>>(                             \
+      g->xs, rv.nbr, rv.N, g->k, g->kp, rv.n0, kf, rv.b, f->sigma, f->logdet, f->not_pd, rl)
   switch (type) {
     case GRAPHGP_MATERN12: GGP_PF(GRAPHGP_MATERN12); break;
     case GRAPHGP_MATERN32: GGP_PF(GRAPHGP_MATERN32); break;
@@ -430,9 +397,9 @@ int point_factor_rows(graphgp_graph_t g, graphgp_factor_t f, const KernF& kf, in
     case 12: GGP_TRY(launch_point_pair<12>(type, g, f, kf, rl, rv, s)); return launch_rescue<12>(type, g, f, kf, rl, rv, s);
     case 16: GGP_TRY(launch_point_pair<16>(type, g, f, kf, rl, rv, s)); return launch_rescue<16>(type, g, f, kf, rl, rv, s);
     case 20:
-    case 24:
+    case 24: GGP_TRY(launch_point_oct<24>(type, g, f, kf, rl, rv, s)); return launch_rescue<24>(type, g, f, kf, rl, rv, s);
     case 28:
-    case 32: GGP_TRY(launch_point<32>(type, g, f, kf, rl, rv, s)); return launch_rescue<32>(type, g, f, kf, rl, rv, s);
+    case 32: GGP_TRY(launch_point_oct<32>(type, g, f, kf, rl, rv, s)); return launch_rescue<32>(type, g, f, kf, rl, rv, s);
     default: GGP_TRY(launch_point_wide(type, g, f, kf, rl, rv, s)); return launch_rescue<kWideK>(type, g, f, kf, rl, rv, s);
   }
 }

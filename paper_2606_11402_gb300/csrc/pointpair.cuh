@@ -45,18 +45,23 @@ struct RowForm {
   float sw, one;
 };
 
-// cov_arg of two squared distances.
-template <int KT>
-__device__ __forceinline__ float2 arg_pair(const KernF& kf, float2 d2) {
-  if (KT == GRAPHGP_SQEXP)
-    return __fmul2_rn(__fmul2_rn(__fmul2_rn(two(0.5f), d2), two(kf.inv_ell)), two(kf.inv_ell));
-  float2 y;  // sqrt_newton
+// sqrt_newton of two arguments.
+__device__ __forceinline__ float2 sqrt_pair(float2 d2) {
+  float2 y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.x) : "f"(d2.x));
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.y) : "f"(d2.y));
   y.x = fminf(y.x, 9.2233720e18f);
   y.y = fminf(y.y, 9.2233720e18f);
   const float2 g = __fmul2_rn(d2, y), h = __fmul2_rn(two(0.5f), y);
-  float2 a = __ffma2_rn(__ffma2_rn(make_float2(-g.x, -g.y), g, d2), h, g);
+  return __ffma2_rn(__ffma2_rn(make_float2(-g.x, -g.y), g, d2), h, g);
+}
+
+// cov_arg of two squared distances.
+template <int KT>
+__device__ __forceinline__ float2 arg_pair(const KernF& kf, float2 d2) {
+  if (KT == GRAPHGP_SQEXP)
+    return __fmul2_rn(__fmul2_rn(__fmul2_rn(two(0.5f), d2), two(kf.inv_ell)), two(kf.inv_ell));
+  float2 a = sqrt_pair(d2);
   if (KT == GRAPHGP_MATERN32) a = __fmul2_rn(two(1.7320508075688772f), a);
   if (KT == GRAPHGP_MATERN52) a = __fmul2_rn(two(2.2360679774997896f), a);
   return __fmul2_rn(a, two(kf.inv_ell));
@@ -532,38 +537,58 @@ __device__ __forceinline__ void pair_rescue(PairFactor<K>& f, bool need, float* 
   }
 }
 
-// kappa / s2 and its derivative by the lengthscale, up to the factor
-// theta_scale, of two squared distances (the values of kappa_dkappa_d2).
-template <int KT>
-__device__ __forceinline__ void dentry_pair(const KernF& kf, float2 d2, float2& pe, float2& de) {
-  const float2 a = arg_pair<KT>(kf, d2);
-  const float2 e = make_float2(expf(-a.x), expf(-a.y));
-  pe = e;
-  if (KT == GRAPHGP_SQEXP || KT == GRAPHGP_MATERN12) {
-    de = __fmul2_rn(a, e);
-    return;
-  }
-  const float2 p = __fadd2_rn(two(1.0f), a), aa = __fmul2_rn(a, a);
-  pe = __fmul2_rn(KT == GRAPHGP_MATERN32 ? p : __ffma2_rn(aa, two(1.0f / 3.0f), p), e);
-  de = __fmul2_rn(KT == GRAPHGP_MATERN32 ? aa : __fmul2_rn(aa, p), e);
-}
+// kappa and d kappa / d lengthscale of two squared distances: the operations of
+// kappa_dkappa_d2 on packed pairs.
+struct DPair {
+  float2 k, l;
+};
 
 template <int KT>
-__device__ __forceinline__ double theta_scale(const KernF& kf) {
-  const double s = (double)kf.s2 * (double)kf.inv_ell;
-  return KT == GRAPHGP_SQEXP ? 2.0 * s : KT == GRAPHGP_MATERN52 ? s / 3.0 : s;
+__device__ __forceinline__ DPair dentry_pair(const KernF& kf, float2 d2) {
+  const float2 s2 = two(kf.s2), il = two(kf.inv_ell);
+  if (KT == GRAPHGP_MATERN12) {
+    const float2 r = sqrt_pair(d2), a = __fmul2_rn(r, il);
+    const float2 k = __fmul2_rn(s2, make_float2(expf(-a.x), expf(-a.y)));
+    return DPair{k, __fmul2_rn(__fmul2_rn(__fmul2_rn(k, r), il), il)};
+  }
+  const float2 a = arg_pair<KT>(kf, d2);
+  const float2 e = make_float2(expf(-a.x), expf(-a.y));
+  if (KT == GRAPHGP_SQEXP) {
+    const float2 k = __fmul2_rn(s2, e);
+    return DPair{k, __fmul2_rn(__fmul2_rn(__fmul2_rn(__fmul2_rn(k, d2), il), il), il)};
+  }
+  const float2 p = __fadd2_rn(two(1.0f), a), saa = __fmul2_rn(__fmul2_rn(s2, a), a);
+  if (KT == GRAPHGP_MATERN32)
+    return DPair{__fmul2_rn(__fmul2_rn(s2, p), e), __fmul2_rn(__fmul2_rn(saa, e), il)};
+  const float2 q = __ffma2_rn(__fmul2_rn(a, a), two(1.0f / 3.0f), p);
+  return DPair{__fmul2_rn(__fmul2_rn(s2, q), e),
+               __fmul2_rn(__fmul2_rn(__fmul2_rn(__fmul2_rn(saa, p), e), il), two(1.0f / 3.0f))};
 }
+
+// Running sums of one row of Kbar against both derivatives, one value at a
+// time in the order of the columns.
+struct RowTheta {
+  float s, l;
+  __device__ __forceinline__ void add(float kb, float k, float dl, float inv_s2) {
+    s = __fmaf_rn(__fmul_rn(kb, k), inv_s2, s);
+    l = __fmaf_rn(kb, dl, l);
+  }
+};
 
 // The per-row factor backward, after pair_factor left the lane's rows of L in
 // f and all of them, with the coordinates, in S: g = K_cc^-1 (alpha v_c), then
-// the cotangent of every covariance value against its derivatives.  With
-// u = g - sbar b the pair (a, c) has cotangent Kbar_ac + Kbar_ca = -(u_a b_c +
-// u_c b_a), the diagonal -u_a b_a and (a, i) g_a - 2 sbar b_a.  The values
-// are visited in the factor's blocks; each FP32 sum takes at most 6 terms per
-// accumulator before it is added to the FP64 totals.  The caller scales tl by
-// theta_scale (s2 is already divided out of ts).  Every lane of the warp must
-// call this; `act` says whether the point counts.  S's rows of L are
-// overwritten.
+// Kbar against dkappa/dtheta: the pair (a, c), c < a, takes Kbar_ac + Kbar_ca =
+// (-g_a b_c + sbar b_a b_c) + (-g_c b_a + sbar b_c b_a), the diagonal -g_a b_a +
+// sbar b_a^2, (a, i) g_a - 2 sbar b_a, and Kbar_ii = sbar.  These terms cancel to
+// a small part of their size, so their order is fixed: each row's sum in FP32
+// over its columns in ascending order and (a, i) last (at most k + 1 terms),
+// then added to the FP64 totals.  A lane takes its own rows, two at a time,
+// four columns per step; in the last step of a row the point stands in the
+// column after the diagonal's.  (Sharing a diagonal block's pairs between the
+// lanes and keeping two partial sums per row is 10 % faster but moves the
+// sigma2 component, the worst conditioned, by 1e-6 of the gradient and more.)
+// Every lane of the warp must call this; `act` says whether the point counts.
+// S's rows of L are overwritten.
 template <int K, int KT>
 __device__ __forceinline__ void pair_row_backward(const PairFactor<K>& f, float* S, int r, int k,
                                                   const KernF& kf, float4 xq,
@@ -574,6 +599,7 @@ __device__ __forceinline__ void pair_row_backward(const PairFactor<K>& f, float*
   using PF = PairFactor<K>;
   constexpr int R = K / 2;
   const unsigned full = 0xffffffffu;
+  const float inv_s2 = 1.0f / kf.s2;
   float g[R];
 #pragma unroll
   for (int s = 0; s < R; s++) g[s] = 2 * s + r < k ? alpha * vv[s] : 0.0f;
@@ -604,120 +630,83 @@ __device__ __forceinline__ void pair_row_backward(const PairFactor<K>& f, float*
 #pragma unroll
   for (int a = 1; a < K; a++) sg += a & 1 ? z[a / 2].y : z[a / 2].x;
   if (f.inc) z[0].x -= sg;
-  // u and b in the place of L's rows; the rows' solves are done on both lanes
+  // g and b in the place of L's rows; the solves are done on both lanes
   __syncwarp();
-  float* U = S + 3 * K;
-  float* B = U + K;
+  float* G = S + 3 * K;
+  float* B = G + K;
 #pragma unroll
   for (int c = 0; c < K / 4; c++) {
-    const int c0 = 2 * c, c1 = 2 * c + 1;
-    if (r)
-      *reinterpret_cast<float4*>(B + 4 * c) = make_float4(f.b[c0].x, f.b[c0].y, f.b[c1].x, f.b[c1].y);
-    else
-      *reinterpret_cast<float4*>(U + 4 * c) =
-          make_float4(z[c0].x - sbar * f.b[c0].x, z[c0].y - sbar * f.b[c0].y,
-                      z[c1].x - sbar * f.b[c1].x, z[c1].y - sbar * f.b[c1].y);
+    const float2 u = r ? f.b[2 * c] : z[2 * c], w = r ? f.b[2 * c + 1] : z[2 * c + 1];
+    *reinterpret_cast<float4*>((r ? B : G) + 4 * c) = make_float4(u.x, u.y, w.x, w.y);
   }
   __syncwarp();
-  double dl = 0.0, ds = 0.0, dn = r ? 0.0 : (double)sbar;  // Kbar_ii = sbar
+  double dl = 0.0, ds = r ? 0.0 : (double)sbar, dn = ds;  // Kbar_ii = sbar
 #pragma unroll 1
-  for (int t = 1; 4 * t < k; t++) {
-    const float* Xa = S + 4 * t + r;
-    const float ax = Xa[0], ay = Xa[K], az = Xa[2 * K];
-    const float bx = Xa[2], by = Xa[K + 2], bz = Xa[2 * K + 2];
-    const float2 ua = two(-U[4 * t + r]), ub = two(-U[4 * t + 2 + r]);
-    const float2 ba = two(-B[4 * t + r]), bb = two(-B[4 * t + 2 + r]);
-    float2 sp = two(0.0f), sl = two(0.0f), sq = two(0.0f), sm = two(0.0f);
+  for (int t = 0; 4 * t < k; t++) {
+    float ng[2], ba[2], sba[2], px[2], py[2], pz[2];
+    RowTheta th[2];
+    float kaa[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const int a = 4 * t + 2 * h + r;
+      ng[h] = -G[a];
+      ba[h] = B[a];
+      sba[h] = __fmul_rn(sbar, ba[h]);
+      px[h] = S[a];
+      py[h] = S[K + a];
+      pz[h] = S[2 * K + a];
+      kaa[h] = __fmaf_rn(sba[h], ba[h], __fmul_rn(ng[h], ba[h]));
+      th[h] = RowTheta{kaa[h], 0.0f};
+    }
 #pragma unroll 1
-    for (int c = 0; c < t; c++) {
-      const float4 X = *reinterpret_cast<const float4*>(S + 4 * c);
-      const float4 Y = *reinterpret_cast<const float4*>(S + K + 4 * c);
-      const float4 Z = *reinterpret_cast<const float4*>(S + 2 * K + 4 * c);
-      const float4 Uc = *reinterpret_cast<const float4*>(U + 4 * c);
+    for (int c = 0; c <= t; c++) {
+      float4 X = *reinterpret_cast<const float4*>(S + 4 * c);
+      float4 Y = *reinterpret_cast<const float4*>(S + K + 4 * c);
+      float4 Z = *reinterpret_cast<const float4*>(S + 2 * K + 4 * c);
+      const float4 Gc = *reinterpret_cast<const float4*>(G + 4 * c);
       const float4 Bc = *reinterpret_cast<const float4*>(B + 4 * c);
+      const float2 b0 = make_float2(Bc.x, Bc.y), b1 = make_float2(Bc.z, Bc.w);
+      const float2 g0 = make_float2(-Gc.x, -Gc.y), g1 = make_float2(-Gc.z, -Gc.w);
+      const float2 s0 = __fmul2_rn(two(sbar), b0), s1 = __fmul2_rn(two(sbar), b1);
 #pragma unroll
       for (int h = 0; h < 2; h++) {
-        const float2 x = h ? make_float2(X.z, X.w) : make_float2(X.x, X.y);
-        const float2 y = h ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y);
-        const float2 w = h ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y);
-        const float2 uc = h ? make_float2(Uc.z, Uc.w) : make_float2(Uc.x, Uc.y);
-        const float2 bc = h ? make_float2(Bc.z, Bc.w) : make_float2(Bc.x, Bc.y);
-        float2 pe, de;
-        dentry_pair<KT>(kf, sqdist2(sub2(ax, x), sub2(ay, y), sub2(az, w)), pe, de);
-        float2 kb = __ffma2_rn(ua, bc, __fmul2_rn(uc, ba));
-        sp = __ffma2_rn(kb, pe, sp);
-        sl = __ffma2_rn(kb, de, sl);
-        dentry_pair<KT>(kf, sqdist2(sub2(bx, x), sub2(by, y), sub2(bz, w)), pe, de);
-        kb = __ffma2_rn(ub, bc, __fmul2_rn(uc, bb));
-        sq = __ffma2_rn(kb, pe, sq);
-        sm = __ffma2_rn(kb, de, sm);
+        const int q = c == t ? 2 * h + r : 4;  // column of the diagonal in this step
+        auto at = [&](float4 u, float pt, int i) {
+          const float x = i == 0 ? u.x : i == 1 ? u.y : i == 2 ? u.z : u.w;
+          return i == q ? pt : x;
+        };
+        auto val = [&](int i) {
+          return dentry_pair<KT>(
+              kf, sqdist2(sub2(px[h], make_float2(at(X, xq.x, i), at(X, xq.x, i + 1))),
+                          sub2(py[h], make_float2(at(Y, xq.y, i), at(Y, xq.y, i + 1))),
+                          sub2(pz[h], make_float2(at(Z, xq.z, i), at(Z, xq.z, i + 1)))));
+        };
+        auto cot = [&](float2 gc, float2 bc, float2 sc) {
+          return __fadd2_rn(
+              __ffma2_rn(two(sba[h]), bc, __fmul2_rn(two(ng[h]), bc)),
+              __ffma2_rn(sc, two(ba[h]), __fmul2_rn(gc, two(ba[h]))));
+        };
+        const float2 k0 = cot(g0, b0, s0), k1 = cot(g1, b1, s1);
+        const float kci = __fmaf_rn(-2.0f * sbar, ba[h], -ng[h]);
+        const DPair d0 = val(0), d1 = val(2);
+        auto pick = [&](float kb, int i) { return i < q ? kb : (i == q ? kci : 0.0f); };
+        th[h].add(pick(k0.x, 0), d0.k.x, d0.l.x, inv_s2);
+        th[h].add(pick(k0.y, 1), d0.k.y, d0.l.y, inv_s2);
+        th[h].add(pick(k1.x, 2), d1.k.x, d1.l.x, inv_s2);
+        th[h].add(pick(k1.y, 3), d1.k.y, d1.l.y, inv_s2);
       }
     }
-    // rows past k have u = b = 0, but their distances may not be finite
-    const bool ra = 4 * t + r < k, rb = 4 * t + 2 + r < k;
-    ds += (ra ? (double)(sp.x + sp.y) : 0.0) + (rb ? (double)(sq.x + sq.y) : 0.0);
-    dl += (ra ? (double)(sl.x + sl.y) : 0.0) + (rb ? (double)(sm.x + sm.y) : 0.0);
-  }
-#pragma unroll 1
-  for (int t = 0; 4 * t < k; t++) {  // diagonal blocks: lane 0's pairs (1, 0) (2, 0) (3, 0) ...
-    const float4 X = *reinterpret_cast<const float4*>(S + 4 * t);
-    const float4 Y = *reinterpret_cast<const float4*>(S + K + 4 * t);
-    const float4 Z = *reinterpret_cast<const float4*>(S + 2 * K + 4 * t);
-    const float4 Ut = *reinterpret_cast<const float4*>(U + 4 * t);
-    const float4 Bt = *reinterpret_cast<const float4*>(B + 4 * t);
-    // ... lane 1's (2, 1) (3, 1) (3, 2); then (2 r, i) (2 r + 1, i)
-#define GGP_LO(q) make_float2(r ? q.y : q.x, r ? q.y : q.x)
-#define GGP_HI(q) make_float2(r ? q.z : q.y, r ? q.w : q.z)
-#define GGP_L2(q) make_float2(r ? q.z : q.x, 0.0f)
-#define GGP_H2(q) make_float2(q.w, 0.0f)
-#define GGP_OWN(q) make_float2(r ? q.z : q.x, r ? q.w : q.y)
-#define GGP_DIST(f, g)                                                                     \
-  sqdist2(make_float2(f(X).x - g(X).x, f(X).y - g(X).y), make_float2(f(Y).x - g(Y).x, f(Y).y - g(Y).y), \
-          make_float2(f(Z).x - g(Z).x, f(Z).y - g(Z).y))
-    float2 pe, de, sp, sl;
-    dentry_pair<KT>(kf, GGP_DIST(GGP_HI, GGP_LO), pe, de);
-    float2 kb = __ffma2_rn(GGP_HI(Ut), GGP_LO(Bt), __fmul2_rn(GGP_LO(Ut), GGP_HI(Bt)));
-    const int hi0 = 4 * t + (r ? 2 : 1), hi1 = hi0 + 1, own0 = 4 * t + 2 * r;
-    kb = make_float2(hi0 < k ? -kb.x : 0.0f, hi1 < k ? -kb.y : 0.0f);
-    if (hi0 >= k) pe.x = de.x = 0.0f;
-    if (hi1 >= k) pe.y = de.y = 0.0f;
-    sp = __fmul2_rn(kb, pe);
-    sl = __fmul2_rn(kb, de);
-    dentry_pair<KT>(kf, GGP_DIST(GGP_H2, GGP_L2), pe, de);
-    if (4 * t + 3 < k) {
-      const float kc = -(Ut.w * GGP_L2(Bt).x + GGP_L2(Ut).x * Bt.w);
-      sp.x = fmaf(kc, pe.x, sp.x);
-      sl.x = fmaf(kc, de.x, sl.x);
-    }
-    const float2 uo = GGP_OWN(Ut), bo = GGP_OWN(Bt), xo = GGP_OWN(X), yo = GGP_OWN(Y),
-                 zo = GGP_OWN(Z);
-    dentry_pair<KT>(kf, sqdist2(sub2(xq.x, xo), sub2(xq.y, yo), sub2(xq.z, zo)), pe, de);
-    float sd = 0.0f;
-    if (own0 < k) {  // g - 2 sbar b = u - sbar b
-      const float kc = fmaf(-sbar, bo.x, uo.x);
-      sp.x = fmaf(kc, pe.x, sp.x);
-      sl.x = fmaf(kc, de.x, sl.x);
-      sd = -uo.x * bo.x;
-    }
-    if (own0 + 1 < k) {
-      const float kc = fmaf(-sbar, bo.y, uo.y);
-      sp.y = fmaf(kc, pe.y, sp.y);
-      sl.y = fmaf(kc, de.y, sl.y);
-      sd = fmaf(-uo.y, bo.y, sd);
-    }
-#undef GGP_LO
-#undef GGP_HI
-#undef GGP_L2
-#undef GGP_H2
-#undef GGP_OWN
-#undef GGP_DIST
-    ds += (double)(sp.x + sp.y);
-    dl += (double)(sl.x + sl.y);
-    dn += (double)sd;
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+      if (4 * t + 2 * h + r < k) {
+        dl += th[h].l;
+        ds += th[h].s;
+        dn += kaa[h];
+      }
   }
   if (act) {
     tl += dl;
-    ts += ds + dn;
+    ts += ds;
     tn += dn;
   }
 }
