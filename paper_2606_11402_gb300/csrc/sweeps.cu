@@ -12,12 +12,15 @@
 // at both ends of the sweep hold a few dozen to a few hundred points (about
 // 90 levels at any N); each of those runs is done by a single block that
 // synchronises with __syncthreads, since a grid barrier per level costs
-// more than the level's work there.
+// more than the level's work there: the first run with its field in shared
+// memory, the last with gathers from L2.  Clouds of at most kFlowEntries row
+// entries have no barrier after the first run: a gathered value is its own flag.
 //
 // whiten: xi_i = (v_i - b_i . v_c(i)) / sigma_i has no dependencies.  Blocks
 // walk spatial tiles through every level (plus xi_0 = L0^-1 v_0 for the
 // dense block), so the gathered v lines of a tile stay in L1; rows are
-// streamed without L1 allocation, v is kept in L2 (evict-last).
+// streamed without L1 allocation, v is kept in L2 (evict-last).  With fewer
+// than four tiles per SM the positions are taken in order by all blocks.
 #include <algorithm>
 
 #include "sweepsync.cuh"
@@ -236,24 +239,309 @@ __global__ void __launch_bounds__(small_threads(KP / LANES), 1) generate_small_k
       nbr, b, sigma, xi, v, level_off, l_first, l_end, n0, none, nullptr);
 }
 
+// ---- the first levels of generate in one block ------------------------------------
+// The levels up to the first large one hold a few dozen to a few hundred points
+// each, and their neighbours are all among the first few ten thousand positions:
+// one block keeps that part of the field in shared memory, so a level costs a
+// block barrier and a shared-memory gather instead of a round trip through L2.
+// Row slices, sigma and xi are loaded D steps ahead, across level boundaries.
+// Bound by the chain barrier - gather - shuffle - store of each level.
+// generate against one block that gathers from L2 and a grid barrier for every
+// level above kTail: 46.4 -> 29.7 us (4096 points, k = 8), 66.9 -> 39.1 (4096,
+// k = 16), 88.4 -> 59.2 (10007, k = 16), 220 -> 188 (127001, k = 16).
+constexpr int kHeadThreads = 512;
+constexpr int64_t kHeadPoints = 49152;  // positions held (192 KB)
+constexpr int kHeadLevels = 4096;
+__host__ __device__ constexpr int head_depth(int hp) { return hp <= 4 ? 3 : (hp <= 8 ? 2 : 1); }
+
+template <int KP, int LANES>
+__global__ void __launch_bounds__(kHeadThreads, 1) generate_head_kernel(
+    const int32_t* __restrict__ nbr, const float* __restrict__ b, const float* __restrict__ sigma,
+    const float* __restrict__ xi, float* __restrict__ v, const int64_t* __restrict__ level_off,
+    int l_end, int64_t n0) {
+  constexpr int HP = KP / LANES, PPB = kHeadThreads / LANES, D = head_depth(HP);
+  extern __shared__ float s_v[];  // the field up to the last level's end, then the offsets
+  const int32_t end = (int32_t)level_off[l_end];
+  int32_t* s_lo = reinterpret_cast<int32_t*>(s_v + end);
+  for (int l = threadIdx.x; l <= l_end; l += kHeadThreads) s_lo[l] = (int32_t)level_off[l];
+  for (int i = threadIdx.x; i < (int)n0; i += kHeadThreads) s_v[i] = v[i];
+  __syncthreads();
+  const int h = threadIdx.x % LANES, slot = threadIdx.x / LANES;
+  const uint64_t pol = l2_policy<0>();
+  const int32_t* nb = nbr + h * HP;
+  const float* bw = b + h * HP;
+  Row<HP> r[D + 1];
+  float sg[D + 1], x[D + 1];
+  // step: level l, first position p; load into buffer i
+  int ll = 1, lp = s_lo[1];  // the next step to load
+  auto load = [&](Row<HP>& row, float& s, float& xv) {
+    if (ll >= l_end) return;
+    const int q = lp + slot;
+    s = xv = 0.0f;
+    if (q < s_lo[ll + 1]) {
+      load_row<HP>(row, nb, bw, ((int64_t)q - n0) * LANES, pol);
+      if (h == 0) {
+        s = ld_stream_f(sigma + q, pol);
+        xv = ld_stream_f(xi + q, pol);
+      }
+    }
+    lp += PPB;
+    if (lp >= s_lo[ll + 1]) lp = s_lo[++ll];
+  };
+#pragma unroll
+  for (int i = 0; i < D; i++) load(r[i], sg[i], x[i]);
+  int l = 1, p = s_lo[1];
+  while (l < l_end) {
+#pragma unroll
+    for (int i = 0; i <= D; i++) {  // buffer i holds this step, i + D is refilled
+      if (l >= l_end) break;
+      load(r[(i + D) % (D + 1)], sg[(i + D) % (D + 1)], x[(i + D) % (D + 1)]);
+      if (p == s_lo[l]) __syncthreads();  // the levels before are complete
+      const int q = p + slot;
+      const bool act = q < s_lo[l + 1];
+      float a0 = 0.0f, a1 = 0.0f;  // gather_dot's order
+      if (act) {
+#pragma unroll
+        for (int c = 0; c < HP / 4; c++) {
+          a0 = fmaf(r[i].w[c].x, s_v[r[i].n[c].x], a0);
+          a1 = fmaf(r[i].w[c].y, s_v[r[i].n[c].y], a1);
+          a0 = fmaf(r[i].w[c].z, s_v[r[i].n[c].z], a0);
+          a1 = fmaf(r[i].w[c].w, s_v[r[i].n[c].w], a1);
+        }
+      }
+      float acc = a0 + a1;
+      if (LANES >= 4) acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+      if (LANES >= 2) acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+      if (act && h == 0) {
+        const float out = fmaf(sg[i], x[i], acc);
+        s_v[q] = out;
+        v[q] = out;
+      }
+      p += PPB;
+      if (p >= s_lo[l + 1]) p = s_lo[++l];
+    }
+  }
+}
+
+// ---- generate by dataflow ------------------------------------------------------
+// Small and medium clouds: no barrier between levels.  v starts as the all-ones
+// NaN (0xffffffff; a NaN result of the arithmetic is the canonical 0x7fffffff,
+// and a store maps the one to the other all the same), and a gathered entry that
+// still holds it is read again at L2 until its value is there: the value is its own flag, so
+// a level costs one trip through L2 instead of a barrier and a gather behind it.
+// Every warp takes its own slice of each level (slices of consecutive warps lie
+// on different SMs, so a level of a few hundred points is spread over as many),
+// in level order and without waiting for the other warps of its block, and
+// loads the rows of its next step, of whichever level, before it gathers the
+// current one.  A cooperative launch: all warps are resident, and the lowest
+// unfinished level never waits for a later one.  Waits are bounded as in the
+// level barrier (a warp may wait here for many levels, so it gets kFlowPolls
+// polls more for each).  Large levels gather most values from L1 behind the
+// barrier, which a flag read at L2 cannot, so they keep the barrier
+// (launch_generate has the line and both sides).
+constexpr uint32_t kNotYet = 0xffffffffu;
+constexpr int kFlowMaxLevels = 4096;  // level table in shared memory
+constexpr int64_t kFlowEntries = 8 << 20;  // N times the padded row length
+constexpr int64_t kFlowPolls = 1024;
+
+__device__ __forceinline__ uint32_t ld_flag(const float* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_flag(float* p, float v) {
+  uint32_t u = __float_as_uint(v);
+  if (u == kNotYet) u = 0x7fffffffu;
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(u) : "memory");
+}
+
+template <int KP, int LANES, int U>
+__global__ void __launch_bounds__(kSweepThreads) generate_flow_kernel(
+    const int32_t* __restrict__ nbr, const float* __restrict__ b, const float* __restrict__ sigma,
+    const float* __restrict__ xi, float* v, const int64_t* __restrict__ level_off, int l_first,
+    int num_levels, int64_t n0, int64_t max_spin, uint32_t* err) {
+  constexpr int HP = KP / LANES, PPW = 32 / LANES;  // row entries per lane, positions per warp
+  extern __shared__ int32_t s_lo[];                 // [num_levels + 1], then slice lengths
+  int32_t* s_per = s_lo + num_levels + 1;
+  const int warps = gridDim.x * (kSweepThreads / 32);
+  for (int l = threadIdx.x; l <= num_levels; l += kSweepThreads) s_lo[l] = (int32_t)level_off[l];
+  __syncthreads();
+  for (int l = threadIdx.x; l < num_levels; l += kSweepThreads) {
+    const uint32_t n = (uint32_t)(s_lo[l + 1] - s_lo[l]);
+    const uint32_t per = (n + warps - 1) / warps;
+    s_per[l] = (int32_t)((per + PPW - 1) / PPW * PPW);
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, h = lane % LANES, grp = lane / LANES;
+  const int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const uint64_t pol = l2_policy<0>();
+  const int32_t* nb = nbr + h * HP;
+  const float* bw = b + h * HP;
+  struct Step {
+    int l;
+    int64_t p, end;
+  };
+  auto first_of = [&](int l) {  // the warp's first step in level l or later
+    for (; l < num_levels; l++) {
+      const int64_t off = (int64_t)w * s_per[l];
+      const int64_t n = s_lo[l + 1] - s_lo[l];
+      if (off < n) return Step{l, s_lo[l] + off, s_lo[l] + min(off + s_per[l], n)};
+    }
+    return Step{l, 0, 0};
+  };
+  Row<HP> rn[U];
+  float sgn[U], xn[U];
+  auto load = [&](const Step& st) {
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int64_t q = st.p + u * PPW + grp;
+      sgn[u] = xn[u] = 0.0f;
+      if (q < st.end) {
+        load_row<HP>(rn[u], nb, bw, (q - n0) * LANES, pol);
+        if (h == 0) {
+          sgn[u] = ld_stream_f(sigma + q, pol);
+          xn[u] = ld_stream_f(xi + q, pol);
+        }
+      }
+    }
+  };
+  Step cur = first_of(l_first);
+  if (cur.l >= num_levels) return;
+  load(cur);
+  while (true) {
+    Row<HP> r[U];
+    float sg[U], x[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      r[u] = rn[u];
+      sg[u] = sgn[u];
+      x[u] = xn[u];
+    }
+    Step nxt = cur;
+    nxt.p += U * PPW;
+    if (nxt.p >= nxt.end) nxt = first_of(cur.l + 1);
+    const bool more = nxt.l < num_levels;
+    if (more) load(nxt);
+    float acc[U];
+    bool dead = false;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      acc[u] = 0.0f;
+      if (cur.p + u * PPW + grp < cur.end) {
+        uint32_t g[HP];
+#pragma unroll
+        for (int q = 0; q < HP / 4; q++) {
+          g[4 * q] = ld_flag(v + r[u].n[q].x);
+          g[4 * q + 1] = ld_flag(v + r[u].n[q].y);
+          g[4 * q + 2] = ld_flag(v + r[u].n[q].z);
+          g[4 * q + 3] = ld_flag(v + r[u].n[q].w);
+        }
+        int64_t spins = 0;
+        while (true) {
+          bool wait = false;
+#pragma unroll
+          for (int q = 0; q < HP; q++) wait |= g[q] == kNotYet;
+          if (!wait || dead) break;
+#pragma unroll
+          for (int q = 0; q < HP / 4; q++) {
+            if (g[4 * q] == kNotYet) g[4 * q] = ld_flag(v + r[u].n[q].x);
+            if (g[4 * q + 1] == kNotYet) g[4 * q + 1] = ld_flag(v + r[u].n[q].y);
+            if (g[4 * q + 2] == kNotYet) g[4 * q + 2] = ld_flag(v + r[u].n[q].z);
+            if (g[4 * q + 3] == kNotYet) g[4 * q + 3] = ld_flag(v + r[u].n[q].w);
+          }
+          __nanosleep(20);
+          if ((++spins & 63) == 0) {
+            if (spins > max_spin) atomicOr(err, ERRBIT_TIMEOUT);
+            dead = sync_ld_acquire(err) & ERRBIT_TIMEOUT;
+          }
+        }
+        float a0 = 0.0f, a1 = 0.0f;  // gather_dot's order
+#pragma unroll
+        for (int q = 0; q < HP / 4; q++) {
+          a0 = fmaf(r[u].w[q].x, __uint_as_float(g[4 * q]), a0);
+          a1 = fmaf(r[u].w[q].y, __uint_as_float(g[4 * q + 1]), a1);
+          a0 = fmaf(r[u].w[q].z, __uint_as_float(g[4 * q + 2]), a0);
+          a1 = fmaf(r[u].w[q].w, __uint_as_float(g[4 * q + 3]), a1);
+        }
+        acc[u] = a0 + a1;
+      }
+    }
+    if (__any_sync(0xffffffffu, dead)) return;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      if (LANES >= 4) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], 2);
+      if (LANES >= 2) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], 1);
+      const int64_t q = cur.p + u * PPW + grp;
+      if (q < cur.end && h == 0) st_flag(v + q, fmaf(sg[u], x[u], acc[u]));
+    }
+    if (!more) return;
+    cur = nxt;
+  }
+}
+
 template <int KP>
-__global__ void __launch_bounds__(256) whiten_kernel(
+int launch_generate_flow(graphgp_graph_t g, graphgp_factor_t f, const float* xi, float* v,
+                         int l_first, cudaStream_t s) {
+  constexpr int LANES = gen_lanes(KP), HP = KP / LANES, U = HP <= 4 ? 2 : 1;
+  int L = g->num_levels;
+  int64_t n0 = g->n0, spin = g->max_spin + kFlowPolls * L;
+  const int64_t p0 = g->level_off_h[l_first];
+  GGP_CUDA(cudaMemsetAsync(v + p0, 0xff, (g->N - p0) * sizeof(float), s));
+  auto kern = generate_flow_kernel<KP, LANES, U>;
+  const size_t smem = (2 * (size_t)L + 1) * sizeof(int32_t);
+  static int max_grid_dev[kMaxDevices] = {};
+  const int max_grid = coop_grid_cached(max_grid_dev, kern, kSweepThreads,
+                                        (2 * (size_t)kFlowMaxLevels + 1) * sizeof(int32_t));
+  // one position per lane group of the largest level is as wide as it gets
+  const int64_t want = (g->max_level_size * LANES + kSweepThreads - 1) / kSweepThreads;
+  const int grid = (int)std::min<int64_t>(max_grid, std::max<int64_t>(want, 1));
+  const int32_t* nbr = g->nbr;
+  const float *bw = f->b, *sg = f->sigma;
+  const int64_t* lod = g->level_off_d;
+  uint32_t* err = g->err;
+  void* args[] = {(void*)&nbr, (void*)&bw, (void*)&sg, (void*)&xi,   (void*)&v,
+                  (void*)&lod, (void*)&l_first, (void*)&L, (void*)&n0, (void*)&spin, (void*)&err};
+  GGP_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(kSweepThreads), args,
+                                       smem, s));
+  return GRAPHGP_OK;
+}
+
+// whiten in position order, LANES lanes per position and U positions per lane
+// group and step.  Bound by DRAM once the rows exceed L2 (10^6 points, k = 16:
+// 140 MB in 60 us) and by latency below.
+template <int KP, int LANES, int U>
+__global__ void __launch_bounds__(256) whiten_flat_kernel(
     const int32_t* __restrict__ nbr, const float* __restrict__ b, const float* __restrict__ sigma,
     const float* __restrict__ v, float* __restrict__ xi, int64_t N, int64_t n0,
     double* __restrict__ sq) {
-  const uint64_t pol_rows = l2_policy<0>();  // whiten: rows evict-normal (measured best)
+  constexpr int HP = KP / LANES, GPB = 256 / LANES;
+  const uint64_t pol_rows = l2_policy<0>();
   const uint64_t pol_v = l2_evict_last();
+  const int h = threadIdx.x % LANES;
   double local = 0.0;
-  for (int64_t pos = n0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; pos < N;
-       pos += (int64_t)gridDim.x * blockDim.x) {
-    Row<KP> r;
-    load_row<KP>(r, nbr, b, pos - n0, pol_rows);
-    float sg = ld_stream_f(sigma + pos, pol_rows);
-    float vi = ld_keep_f(v + pos, pol_v);
-    float acc = gather_dot<KP, false>(r, v, pol_v);
-    float out = (vi - acc) / sg;
-    st_stream_f(xi + pos, out, pol_rows);
-    if (sq) local += (double)out * (double)out;
+  for (int64_t p0 = n0 + (int64_t)blockIdx.x * (GPB * U) + threadIdx.x / LANES;
+       p0 - threadIdx.x / LANES < N; p0 += (int64_t)gridDim.x * (GPB * U)) {
+    Row<HP> r[U];
+    float acc[U];
+#pragma unroll
+    for (int u = 0; u < U; u++)
+      if (p0 + u * GPB < N)
+        load_row_na<HP>(r[u], nbr + h * HP, b + h * HP, (p0 + u * GPB - n0) * LANES, pol_rows);
+#pragma unroll
+    for (int u = 0; u < U; u++)
+      acc[u] = p0 + u * GPB < N ? gather_dot<HP, false>(r[u], v, pol_v) : 0.0f;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      if (LANES >= 4) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], 2);
+      if (LANES >= 2) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], 1);
+      const int64_t pos = p0 + u * GPB;
+      if (pos < N && h == 0) {
+        const float out = (ld_keep_f(v + pos, pol_v) - acc[u]) / ld_stream_na_f(sigma + pos, pol_rows);
+        st_stream_f(xi + pos, out, pol_rows);
+        if (sq) local += (double)out * (double)out;
+      }
+    }
   }
   if (sq) {
     __shared__ double red[8];
@@ -373,23 +661,34 @@ int launch_generate(graphgp_graph_t g, graphgp_factor_t f, const float* xi, floa
   const int L = g->num_levels;
   if (L <= 1) return GRAPHGP_OK;
   constexpr int LANES = gen_lanes(KP), HP = KP / LANES, U = gen_steps(HP);
-  // Runs of small levels at both ends of the sweep (a level that one block
-  // covers in two steps) go to one block; the levels between them to the
-  // cooperative grid.  Levels [1, a) and [z, L) are small.
-  constexpr int64_t kSmall = 2 * small_steps(HP) * (small_threads(HP) / LANES);
+  // The run of small levels that the sweep starts with (a level that one block
+  // covers in a few steps) goes to one block with its field in shared memory.
+  constexpr int64_t kSmall = 1024;
   const std::vector<int64_t>& lo = g->level_off_h;
   int a = 1;
-  while (a < L && lo[a + 1] - lo[a] <= kSmall) a++;
-  int z = L;
-  while (z > a && lo[z] - lo[z - 1] <= kSmall) z--;
+  while (a < L && a < kHeadLevels && lo[a + 1] - lo[a] <= kSmall && lo[a + 1] <= kHeadPoints) a++;
   const int64_t* lod = g->level_off_d;
   int64_t n0 = g->n0;
-  constexpr int NTS = small_threads(HP);
   if (a > 1) {
-    generate_small_kernel<KP, LANES><<<1, NTS, 0, s>>>(g->nbr, f->b, f->sigma, xi, v, lod, 1, a,
-                                                       n0);
+    const size_t smem = (size_t)lo[a] * sizeof(float) + (a + 1) * sizeof(int32_t);
+    auto kern = generate_head_kernel<KP, LANES>;
+    GGP_CUDA(allow_dyn_smem(kern, smem));
+    kern<<<1, kHeadThreads, smem, s>>>(g->nbr, f->b, f->sigma, xi, v, lod, a, n0);
     GGP_CUDA(cudaGetLastError());
   }
+  if (a == L) return GRAPHGP_OK;
+  // Without a barrier up to kFlowEntries row entries (barrier / flags, us): 30011
+  // points, k = 16: 125 / 104; 127001, k = 7: 99 / 76; 10^6, k = 8: 168 / 143;
+  // 500000, k = 16: 252 / 212; 262000, k = 32: 469 / 356; 130000, k = 64: 1058 /
+  // 851.  Above, the values are no longer read soon after they are written: 10^6,
+  // k = 16: 286 / 294, k = 32: 603 / 1217; 2^24, k = 16: 902 / 1098.
+  const bool flow = g->N * KP <= kFlowEntries && L <= kFlowMaxLevels;
+  if (flow) return launch_generate_flow<KP>(g, f, xi, v, a, s);
+  // the levels in between to the cooperative grid, the run of small ones at the
+  // end (levels [z, L)) to one block
+  constexpr int64_t kTail = 2 * small_steps(HP) * (small_threads(HP) / LANES);
+  int z = L;
+  while (z > a && lo[z] - lo[z - 1] <= kTail) z--;
   if (a < z) {
     GGP_CUDA(cudaMemsetAsync(g->level_bar, 0, L * sizeof(uint32_t), s));
     auto kern = generate_kernel<KP, LANES, U>;
@@ -407,8 +706,8 @@ int launch_generate(graphgp_graph_t g, graphgp_factor_t f, const float* xi, floa
                                          0, s));
   }
   if (z < L) {
-    generate_small_kernel<KP, LANES><<<1, NTS, 0, s>>>(g->nbr, f->b, f->sigma, xi, v, lod, z, L,
-                                                       n0);
+    generate_small_kernel<KP, LANES><<<1, small_threads(HP), 0, s>>>(g->nbr, f->b, f->sigma, xi, v,
+                                                                     lod, z, L, n0);
     GGP_CUDA(cudaGetLastError());
   }
   return GRAPHGP_OK;
@@ -419,7 +718,12 @@ int launch_whiten(graphgp_graph_t g, graphgp_factor_t f, const float* v, float* 
                   cudaStream_t s) {
   int64_t n = g->N - g->n0;
   if (n <= 0) return GRAPHGP_OK;
-  if (g->tile_start && g->num_levels <= 8192) {
+  // A tile is one block's work, so fewer than four per SM leave the chip idle or
+  // its last wave nearly empty (tiles / in order, us; k = 16): 4096 points 74 / 16,
+  // 10^6 136 / 60, 2^21 (3.4 tiles per SM) 143 / 104; 2^22 (6.7 per SM) 166 / 188,
+  // k = 8 92 / 98; 2^24 601 / 726: there the tile's gathers from L1 win.
+  const bool tiled = g->n_tiles >= 4 * (int64_t)num_sms();
+  if (tiled && g->tile_start && g->num_levels <= 8192) {
     size_t smem = (2 * (size_t)g->num_levels + 1) * sizeof(int32_t);
     GGP_CUDA(allow_dyn_smem(whiten_tiles_kernel<KP>, smem));
     int per_sm = 0;
@@ -428,8 +732,11 @@ int launch_whiten(graphgp_graph_t g, graphgp_factor_t f, const float* v, float* 
     whiten_tiles_kernel<KP><<<(unsigned)grid, 256, smem, s>>>(
         g->nbr, f->b, f->sigma, v, xi, g->n0, g->tile_start, g->n_tiles, g->num_levels, sq);
   } else {
-    whiten_kernel<KP><<<grid_for(n, 256, 8), 256, 0, s>>>(g->nbr, f->b, f->sigma, v, xi, g->N,
-                                                          g->n0, sq);
+    constexpr int LANES = gen_lanes(KP), U = KP / LANES <= 4 ? 2 : 1;
+    const int64_t per = 256 / LANES * U;
+    const int64_t grid = std::min<int64_t>((n + per - 1) / per, (int64_t)num_sms() * 8);
+    whiten_flat_kernel<KP, LANES, U><<<(unsigned)grid, 256, 0, s>>>(g->nbr, f->b, f->sigma, v, xi,
+                                                                    g->N, g->n0, sq);
   }
   GGP_CUDA(cudaGetLastError());
   return GRAPHGP_OK;
