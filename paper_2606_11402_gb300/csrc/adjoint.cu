@@ -30,14 +30,41 @@ namespace ggp {
 namespace {
 
 // ---- dense helpers ------------------------------------------------------------
-// y_m = sum_{i >= m} M[i][m] x_i (transpose of a lower-triangular n0 x n0 M)
-__global__ void dense_lower_tmatvec_kernel(const float* __restrict__ M, const float* __restrict__ x,
-                                           float* __restrict__ y, int n0) {
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n0; m += gridDim.x * blockDim.x) {
-    float s = 0.0f;
-    for (int i = m; i < n0; i++) s = fmaf(M[(int64_t)i * n0 + m], x[i], s);
-    y[m] = s;
+// y_m (+)= sum_{i >= m} M[i][m] x_i (transpose of a lower-triangular n0 x n0 M).
+// A block takes 32 columns: its warps stage kTmvRows rows of them at once, then
+// one warp adds down the columns, so that the sum keeps its order (ascending i,
+// one accumulator).  Bound by that chain and two memory latencies per chunk; a
+// thread per column waited for one load after another: n0 = 256
+// 66 -> 5.3 us.
+constexpr int kTmvRows = 256;
+
+template <bool ACC>
+__global__ void __launch_bounds__(256) dense_lower_tmatvec_kernel(
+    const float* __restrict__ M, const float* __restrict__ x, float* __restrict__ y, int n0) {
+  __shared__ float s_m[kTmvRows][32], s_x[kTmvRows];
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5, m0 = blockIdx.x * 32, m = m0 + c;
+  float s = 0.0f;
+  for (int i0 = m0; i0 < n0; i0 += kTmvRows) {
+    const int rows = min(kTmvRows, n0 - i0);
+    float r[kTmvRows / 8];
+#pragma unroll
+    for (int t = 0; t < kTmvRows / 8; t++) {
+      const int i = i0 + w + 8 * t;
+      r[t] = (i < n0 && m < n0) ? M[(int64_t)i * n0 + m] : 0.0f;
+    }
+    const float xr = (int)threadIdx.x < rows ? x[i0 + threadIdx.x] : 0.0f;
+    __syncthreads();  // the chunk before has been read
+#pragma unroll
+    for (int t = 0; t < kTmvRows / 8; t++) s_m[w + 8 * t][c] = r[t];
+    s_x[threadIdx.x] = xr;
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll 16
+      for (int t = 0; t < rows; t++)
+        if (i0 + t >= m) s = fmaf(s_m[t][c], s_x[t], s);
+    }
   }
+  if (w == 0 && m < n0) y[m] = ACC ? y[m] + s : s;
 }
 
 // Lbar0[a][b] = sgn * u_a xi_b (b <= a) plus diag 2 logdetbar / L0_aa.
@@ -54,24 +81,72 @@ __global__ void dense_lbar_kernel(const float* __restrict__ u, const float* __re
   }
 }
 
-// C = op(A) B for n x n row-major matrices; op(A) = A^T when transA.  If phi,
-// keeps the lower triangle of the result with the diagonal halved.
-__global__ void dense_gemm_kernel(const float* __restrict__ A, const float* __restrict__ B,
-                                  float* __restrict__ C, int n, int transA, int phi) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)n * n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int a = (int)(e / n), b = (int)(e % n);
-    if (phi && b > a) {
-      C[e] = 0.0f;
-      continue;
+// C = op(A) B for n x n row-major matrices; op(A) = A^T when TRANS.  If PHI,
+// keeps the lower triangle of the result with the diagonal halved.  32 x 32 of C
+// per block from 32-row chunks of both operands in shared memory, the next chunk
+// loaded meanwhile; a thread has four neighbouring entries, each one accumulator
+// over ascending m.  At n = 256 there are 64 tiles, so a chunk's latency bounds
+// it; a thread per entry that read both operands from L2
+// took 34 us (n = 256), this 10-13 us.
+constexpr int kGemmTile = 32;
+
+template <bool TRANS, bool PHI>
+__global__ void __launch_bounds__(256) dense_gemm_kernel(const float* __restrict__ A,
+                                                         const float* __restrict__ B,
+                                                         float* __restrict__ C, int n) {
+  constexpr int T = kGemmTile;
+  __shared__ float s_a[T][T + 1];              // [m][row of C]
+  __shared__ __align__(16) float s_b[T][T];    // [m][column of C]
+  const int a0 = blockIdx.y * T, b0 = blockIdx.x * T;
+  const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;  // loads: 8 rows of 32
+  const int row = threadIdx.x >> 3, col = (threadIdx.x & 7) * 4;
+  float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  if (!PHI || b0 <= a0) {
+    float ra[4], rb[4];
+    auto load = [&](int m0) {
+#pragma unroll
+      for (int t = 0; t < 4; t++) {
+        const int y = ly + 8 * t, m = m0 + y;
+        if (TRANS)
+          ra[t] = (m < n && a0 + lx < n) ? A[(int64_t)m * n + a0 + lx] : 0.0f;
+        else
+          ra[t] = (a0 + y < n && m0 + lx < n) ? A[(int64_t)(a0 + y) * n + m0 + lx] : 0.0f;
+        rb[t] = (m < n && b0 + lx < n) ? B[(int64_t)m * n + b0 + lx] : 0.0f;
+      }
+    };
+    load(0);
+    for (int m0 = 0; m0 < n; m0 += T) {
+      __syncthreads();  // the chunk before has been read
+#pragma unroll
+      for (int t = 0; t < 4; t++) {
+        const int y = ly + 8 * t;
+        if (TRANS)
+          s_a[y][lx] = ra[t];
+        else
+          s_a[lx][y] = ra[t];
+        s_b[y][lx] = rb[t];
+      }
+      __syncthreads();
+      if (m0 + T < n) load(m0 + T);
+#pragma unroll
+      for (int m = 0; m < T; m++) {
+        const float a = s_a[m][row];
+        const float4 v = *reinterpret_cast<const float4*>(&s_b[m][col]);
+        s[0] = fmaf(a, v.x, s[0]);
+        s[1] = fmaf(a, v.y, s[1]);
+        s[2] = fmaf(a, v.z, s[2]);
+        s[3] = fmaf(a, v.w, s[3]);
+      }
     }
-    float s = 0.0f;
-    if (transA)
-      for (int m = 0; m < n; m++) s = fmaf(A[(int64_t)m * n + a], B[(int64_t)m * n + b], s);
-    else
-      for (int m = 0; m < n; m++) s = fmaf(A[(int64_t)a * n + m], B[(int64_t)m * n + b], s);
-    if (phi && a == b) s *= 0.5f;
-    C[e] = s;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    const int a = a0 + row, b = b0 + col + q;
+    if (a < n && b < n) {
+      float out = s[q];
+      if (PHI) out = b > a ? 0.0f : (a == b ? 0.5f * out : out);
+      C[(int64_t)a * n + b] = out;
+    }
   }
 }
 
@@ -203,13 +278,14 @@ __global__ void __launch_bounds__(256) whiten_adjoint_scatter_kernel(
 template <int KP>
 __global__ void __launch_bounds__(256) generate_adjoint_scatter_kernel(
     const int32_t* __restrict__ nbr, const float* __restrict__ b, float* u,
-    const int64_t* __restrict__ level_off, int num_levels, int64_t n0, LevelBarrier lb) {
+    const int64_t* __restrict__ level_off, int l_first, int num_levels, int64_t n0,
+    LevelBarrier lb) {
   constexpr int LANES = gen_lanes(KP), HP = KP / LANES, GPB = 256 / LANES;
   __shared__ int s_flag;
   const int h = threadIdx.x % LANES;
   const uint64_t pol = l2_evict_first();
   const uint64_t pol_u = l2_evict_last();
-  for (int l = num_levels - 1; l >= 1; l--) {
+  for (int l = num_levels - 1; l >= l_first; l--) {
     const int64_t lo = level_off[l], cnt = level_off[l + 1] - lo;
     const int64_t per = (cnt + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = lo + min((int64_t)blockIdx.x * per, cnt);
@@ -235,6 +311,63 @@ __global__ void __launch_bounds__(256) generate_adjoint_scatter_kernel(
     __syncthreads();
     lb.arrive(l);
   }
+}
+
+// generate VJP, the levels the sweep ends with (the first of the graph, a few
+// dozen points each): one block with u up to their end in shared memory, so a
+// level costs a block barrier and shared-memory atomics instead of a grid barrier
+// and a round trip through L2.  Rows are loaded D steps ahead, across levels.
+// Bound by the shared-memory atomics, so the run ends at the first level with
+// more than kHeadEntries row entries.  The vector-only VJP with no such run / one
+// up to 64 / 128 / 256 / 512 points a level, us: 127001 points, k = 16: 221 / 200 /
+// 192 / 192 / 202; k = 48: 713 / 653 / 641 / 674 / 800; k = 7 (padded to 8): 123 /
+// 126 / 122 / 118 / 118; 10^6, k = 16: 427 / 408 / 390 / 382 / 386.
+constexpr int kHeadThreads = 512;
+constexpr int64_t kHeadPoints = 49152;  // positions held (192 KB)
+constexpr int kHeadLevels = 4096;
+constexpr int64_t kHeadEntries = 4096;  // row entries of its largest level
+
+template <int KP>
+__global__ void __launch_bounds__(kHeadThreads, 1) generate_adjoint_head_kernel(
+    const int32_t* __restrict__ nbr, const float* __restrict__ b, float* __restrict__ u,
+    const int64_t* __restrict__ level_off, int l_end, int64_t n0) {
+  constexpr int LANES = gen_lanes(KP), HP = KP / LANES, PPB = kHeadThreads / LANES;
+  constexpr int D = HP <= 4 ? 3 : (HP <= 8 ? 2 : 1);
+  extern __shared__ float s_u[];  // u up to the last level's end, then the offsets
+  const int32_t end = (int32_t)level_off[l_end];
+  int32_t* s_lo = reinterpret_cast<int32_t*>(s_u + end);
+  for (int l = threadIdx.x; l <= l_end; l += kHeadThreads) s_lo[l] = (int32_t)level_off[l];
+  for (int i = threadIdx.x; i < end; i += kHeadThreads) s_u[i] = u[i];
+  __syncthreads();
+  const int h = threadIdx.x % LANES, slot = threadIdx.x / LANES;
+  const uint64_t pol = l2_policy<0>();
+  int4 n[D + 1][HP / 4];
+  float4 w[D + 1][HP / 4];
+  int ll = l_end - 1, lp = s_lo[ll];  // the next step to load
+  auto load = [&](int4 (&nn)[HP / 4], float4 (&ww)[HP / 4]) {
+    if (ll < 1) return;
+    const int q = lp + slot;
+    if (q < s_lo[ll + 1]) load_row_slice<HP>(nn, ww, nbr, b, ((int64_t)q - n0) * KP + h * HP, pol);
+    lp += PPB;
+    if (lp >= s_lo[ll + 1]) lp = s_lo[--ll];
+  };
+#pragma unroll
+  for (int i = 0; i < D; i++) load(n[i], w[i]);
+  int l = l_end - 1, p = s_lo[l];
+  while (l >= 1) {
+#pragma unroll
+    for (int i = 0; i <= D; i++) {  // buffer i holds this step, i + D is refilled
+      if (l < 1) break;
+      load(n[(i + D) % (D + 1)], w[(i + D) % (D + 1)]);
+      if (p == s_lo[l]) __syncthreads();  // the levels behind are complete
+      const int q = p + slot;
+      if (q < s_lo[l + 1]) scatter_row<HP>(s_u, n[i], w[i], s_u[q]);
+      p += PPB;
+      if (p >= s_lo[l + 1]) p = s_lo[--l];
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < end; i += kHeadThreads) u[i] = s_u[i];
 }
 
 int whiten_adjoint_scatter(graphgp_graph_t g, graphgp_factor_t f, const float* xibar, float* vbar,
@@ -899,9 +1032,10 @@ int dense_kbar(graphgp_graph_t g, graphgp_factor_t f, const float* u0, const flo
   GGP_TRY(sc.alloc(&T, nn));
   unsigned grid = grid_for(nn, 256);
   dense_lbar_kernel<<<grid, 256, 0, s>>>(u0, xi0, f->L0, n0, sgn, ldbar, Kbar);
-  dense_gemm_kernel<<<grid, 256, 0, s>>>(f->L0, Kbar, P, n0, 1, 1);     // Phi(L0^T Lbar0)
-  dense_gemm_kernel<<<grid, 256, 0, s>>>(f->L0inv, P, T, n0, 1, 0);     // L0^-T P
-  dense_gemm_kernel<<<grid, 256, 0, s>>>(T, f->L0inv, Kbar, n0, 0, 0);  // (L0^-T P) L0^-1
+  const dim3 tiles((n0 + kGemmTile - 1) / kGemmTile, (n0 + kGemmTile - 1) / kGemmTile);
+  dense_gemm_kernel<true, true><<<tiles, 256, 0, s>>>(f->L0, Kbar, P, n0);  // Phi(L0^T Lbar0)
+  dense_gemm_kernel<true, false><<<tiles, 256, 0, s>>>(f->L0inv, P, T, n0);  // L0^-T P
+  dense_gemm_kernel<false, false><<<tiles, 256, 0, s>>>(T, f->L0inv, Kbar, n0);  // (L0^-T P) L0^-1
   GGP_CUDA(cudaGetLastError());
   return GRAPHGP_OK;
 }
@@ -935,7 +1069,7 @@ int run_whiten_backward(graphgp_graph_t g, graphgp_factor_t f, const float* v, c
                         cudaStream_t s) {
   int n0 = g->n0;
   // dense: vbar_0 = L0^-T xibar_0 (then children are subtracted below)
-  dense_lower_tmatvec_kernel<<<(n0 + 255) / 256, 256, 0, s>>>(f->L0inv, xibar, vbar, n0);
+  dense_lower_tmatvec_kernel<false><<<(n0 + 31) / 32, 256, 0, s>>>(f->L0inv, xibar, vbar, n0);
   GGP_CUDA(cudaGetLastError());
   if (thetabar) GGP_TRY(dense_backward(g, f, vbar, xi, -1.0f, (float)logdetbar, thetabar, s));
   if (g->N > n0) {
@@ -952,16 +1086,20 @@ int run_generate_backward(graphgp_graph_t g, graphgp_factor_t f, const float* xi
   float* u = g->tmp_vec;
   int n0 = g->n0;
   GGP_CUDA(cudaMemcpyAsync(u, vbar, g->N * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  if (g->num_levels > 1) {
+  const std::vector<int64_t>& lo = g->level_off_h;
+  const int32_t* nb = g->nbr;
+  const float* bw = f->b;
+  const int64_t* lod = g->level_off_d;
+  int nl = g->num_levels, head = 1;  // levels [1, head) to one block
+  int64_t n0l = n0;
+  while (head < nl && head < kHeadLevels && (lo[head + 1] - lo[head]) * g->kp <= kHeadEntries &&
+         lo[head + 1] <= kHeadPoints)
+    head++;
+  if (head < nl) {
     GGP_CUDA(cudaMemsetAsync(g->level_bar, 0, g->num_levels * sizeof(uint32_t), s));
     LevelBarrier lb{g->level_bar, g->err, g->max_spin};
-    const int32_t* nb = g->nbr;
-    const float* bw = f->b;
-    const int64_t* lo = g->level_off_d;
-    int nl = g->num_levels;
-    int64_t n0l = n0;
-    void* args[] = {(void*)&nb, (void*)&bw, (void*)&u, (void*)&lo, (void*)&nl, (void*)&n0l,
-                    (void*)&lb};
+    void* args[] = {(void*)&nb, (void*)&bw, (void*)&u, (void*)&lod, (void*)&head, (void*)&nl,
+                    (void*)&n0l, (void*)&lb};
 #define GGP_GSC(KP)                                                                              \
   {                                                                                              \
     static int max_grid_dev[kMaxDevices] = {};                                                   \
@@ -973,8 +1111,19 @@ int run_generate_backward(graphgp_graph_t g, graphgp_factor_t f, const float* xi
     GGP_ADJ_KP_DISPATCH(g->kp, GGP_GSC);
 #undef GGP_GSC
   }
+  if (head > 1) {
+    const size_t smem = (size_t)lo[head] * sizeof(float) + (head + 1) * sizeof(int32_t);
+#define GGP_GSH(KP)                                                                         \
+  {                                                                                         \
+    GGP_CUDA(allow_dyn_smem(generate_adjoint_head_kernel<KP>, smem));                       \
+    generate_adjoint_head_kernel<KP><<<1, kHeadThreads, smem, s>>>(nb, bw, u, lod, head, n0l); \
+  }
+    GGP_ADJ_KP_DISPATCH(g->kp, GGP_GSH);
+#undef GGP_GSH
+    GGP_CUDA(cudaGetLastError());
+  }
   // dense: xibar_0 = L0^T u_0, Lbar0 = tril(u_0 xi_0^T)
-  dense_lower_tmatvec_kernel<<<(n0 + 255) / 256, 256, 0, s>>>(f->L0, u, xibar, n0);
+  dense_lower_tmatvec_kernel<false><<<(n0 + 31) / 32, 256, 0, s>>>(f->L0, u, xibar, n0);
   GGP_CUDA(cudaGetLastError());
   if (!thetabar) {  // vector cotangent only: xibar_i = sigma_i u_i
     if (g->N > n0)
@@ -1036,16 +1185,6 @@ __global__ void whiten_rows_kernel(const int32_t* __restrict__ nbr, const float*
   if (sq) block_add_double(local, sq);
 }
 
-// y[m] += sum_{i >= m} M[i][m] x[i] for the n0 x n0 lower-triangular M.
-__global__ void dense_tmatvec_acc_kernel(const float* __restrict__ M, const float* __restrict__ x,
-                                         float* __restrict__ y, int n0) {
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n0; m += gridDim.x * blockDim.x) {
-    float s = 0.0f;
-    for (int i = m; i < n0; i++) s = fmaf(M[(int64_t)i * n0 + m], x[i], s);
-    y[m] += s;
-  }
-}
-
 __global__ void nll_rows_finish_kernel(const double* __restrict__ sq,
                                        const double* __restrict__ logdet,
                                        double* __restrict__ out) {
@@ -1105,8 +1244,8 @@ extern "C" int graphgp_nll_backward_rows(graphgp_graph_t g, graphgp_factor_t f, 
     Scratch sc(s);
     float* u0 = nullptr;
     GGP_TRY(sc.alloc(&u0, n0));
-    dense_lower_tmatvec_kernel<<<(n0 + 255) / 256, 256, 0, s>>>(f->L0inv, xibar, u0, n0);
-    dense_tmatvec_acc_kernel<<<(n0 + 255) / 256, 256, 0, s>>>(f->L0inv, xibar, vbar_d, n0);
+    dense_lower_tmatvec_kernel<false><<<(n0 + 31) / 32, 256, 0, s>>>(f->L0inv, xibar, u0, n0);
+    dense_lower_tmatvec_kernel<true><<<(n0 + 31) / 32, 256, 0, s>>>(f->L0inv, xibar, vbar_d, n0);
     GGP_CUDA(cudaGetLastError());
     GGP_TRY(dense_backward(g, f, u0, xi, -1.0f, (float)(0.5 * nllbar), thetabar_d, s));
   }
@@ -1178,7 +1317,7 @@ extern "C" int graphgp_nll_grad_fused(graphgp_graph_t g, const graphgp_kernel* k
   GGP_TRY(dense_into(g, kern, sc, acc + 1, bad, f, s));
   GGP_TRY(dense_matvec(f.L0inv, v_d, xi, n0, acc, s));
   scale_kernel<<<(n0 + 255) / 256, 256, 0, s>>>(xi, (float)nllbar, xb, n0);
-  dense_lower_tmatvec_kernel<<<(n0 + 255) / 256, 256, 0, s>>>(f.L0inv, xb, vbar_d, n0);
+  dense_lower_tmatvec_kernel<false><<<(n0 + 31) / 32, 256, 0, s>>>(f.L0inv, xb, vbar_d, n0);
   GGP_CUDA(cudaGetLastError());
   GGP_TRY(dense_backward(g, &f, vbar_d, xi, -1.0f, (float)(0.5 * nllbar), thetabar_d, s));
   if (g->N > n0) {
