@@ -11,6 +11,8 @@
 //     of the left subtree) of that dimension's range: no selection pass;
 //   * the two other orders are stably partitioned (left part, node, right
 //     part) with one exclusive scan each, so they stay sorted.
+// Once a subtree has at most kSub nodes, one block takes it through all of its
+// levels in shared memory (tree_sub_kernel).
 // Every step is a permutation fixed by the data, so the result is exactly
 // the recursive definition: split on the widest FP32 extent (ties to the
 // lowest dimension) or on level mod 3, median by (coordinate, input index).
@@ -23,22 +25,16 @@ __device__ __forceinline__ int node_level(int64_t j) {
   return 63 - __clzll((unsigned long long)(j + 1));
 }
 
-// Number of existing nodes in the subtree of j: the descendants of the node
-// at (level l, position p) on level m occupy positions p + t 2^l, t < 2^(m-l).
-__device__ int64_t subtree_nodes(int64_t j, int64_t N) {
-  if (j >= N) return 0;
-  int l = node_level(j);
-  int64_t p = j - ((int64_t(1) << l) - 1);
-  int64_t stride = int64_t(1) << l;
-  int64_t count = 0;
-  for (int m = l; m < 63; m++) {
-    int64_t lo = (int64_t(1) << m) - 1 + p;
-    if (lo >= N) break;
-    int64_t cap = int64_t(1) << (m - l);
-    int64_t n = (N - lo + stride - 1) / stride;
-    count += n < cap ? n : cap;
-  }
-  return count;
+// Number of existing nodes in the subtree at (level l, position p): the
+// descendants on level m occupy positions p + t 2^l, t < 2^(m-l); every level but
+// the last is full.
+__host__ __device__ __forceinline__ int64_t subtree_nodes(int64_t p, int l, int64_t N, int levels) {
+  if (l >= levels) return 0;
+  const int64_t cap = int64_t(1) << (levels - 1 - l);
+  const int64_t rest = N - ((int64_t(1) << (levels - 1)) - 1 + p);
+  if (rest <= 0) return cap - 1;
+  const int64_t n = ((rest - 1) >> l) + 1;
+  return cap - 1 + (n < cap ? n : cap);
 }
 
 __device__ __forceinline__ uint32_t orderable(float f) {
@@ -63,7 +59,7 @@ struct Orders {
 // One thread per node of level l: split dimension, median point, in-order
 // rank, and the in-order start of both children.
 __global__ void level_nodes_kernel(const float* __restrict__ pts, int64_t N,
-                                   int l, int rule, Orders ord,
+                                   int l, int levels, int rule, Orders ord,
                                    int32_t* __restrict__ start,
                                    int32_t* __restrict__ msize,
                                    int32_t* __restrict__ tree_point,
@@ -77,9 +73,9 @@ __global__ void level_nodes_kernel(const float* __restrict__ pts, int64_t N,
        t += (int64_t)gridDim.x * blockDim.x) {
     int64_t j = first + t;
     if (j >= N) return;
-    int64_t S = subtree_nodes(j, N);
+    int64_t S = subtree_nodes(t, l, N, levels);
     int64_t lc = j + (int64_t(1) << l), rc = j + (int64_t(2) << l);
-    int64_t m = subtree_nodes(lc, N);
+    int64_t m = subtree_nodes(t, l + 1, N, levels);
     int64_t st = start[j];
     int dim;
     float lo[3], hi[3], ext[3];
@@ -142,14 +138,18 @@ __global__ void slot_side_kernel(int64_t N, Orders ord,
   }
 }
 
-// Flags of the elements that go left in the order of dimension A, inside
-// subtrees that do not split on A; records the slot of each node element.
-__global__ void part_flags_kernel(int64_t N, int A, const int32_t* __restrict__ ordA,
-                                  const int32_t* __restrict__ seg,
+// Flags of the elements that go left in the order of dimension A = A0 +
+// blockIdx.y, inside subtrees that do not split on A; records the slot of each
+// node element.  flags and node_slot hold N entries per dimension of the launch.
+__global__ void part_flags_kernel(int64_t N, int A0, Orders ord, const int32_t* __restrict__ seg,
                                   const uint8_t* __restrict__ split_dim,
                                   const uint8_t* __restrict__ side,
                                   uint32_t* __restrict__ flags,
                                   int32_t* __restrict__ node_slot) {
+  const int A = A0 + blockIdx.y;
+  const int32_t* ordA = ord.o[A];
+  flags += blockIdx.y * N;
+  node_slot += blockIdx.y * N;
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < N;
        x += (int64_t)gridDim.x * blockDim.x) {
     int32_t j = seg[x];
@@ -163,9 +163,13 @@ __global__ void part_flags_kernel(int64_t N, int A, const int32_t* __restrict__ 
   }
 }
 
-__global__ void part_scatter_kernel(int64_t N, int A,
-                                    const int32_t* __restrict__ ordA,
-                                    int32_t* __restrict__ ordA_next,
+struct OrdersOut {
+  int32_t* o[3];
+};
+
+// pre: exclusive prefix of flags over all dimensions of the launch; only
+// differences within one dimension are used.
+__global__ void part_scatter_kernel(int64_t N, int A0, Orders ord, OrdersOut next,
                                     const int32_t* __restrict__ seg,
                                     const uint8_t* __restrict__ split_dim,
                                     const uint8_t* __restrict__ side,
@@ -173,6 +177,11 @@ __global__ void part_scatter_kernel(int64_t N, int A,
                                     const int32_t* __restrict__ start,
                                     const int32_t* __restrict__ msize,
                                     const int32_t* __restrict__ node_slot) {
+  const int A = A0 + blockIdx.y;
+  const int32_t* ordA = ord.o[A];
+  int32_t* ordA_next = next.o[A];
+  pre += blockIdx.y * N;
+  node_slot += blockIdx.y * N;
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < N;
        x += (int64_t)gridDim.x * blockDim.x) {
     int32_t j = seg[x];
@@ -181,7 +190,7 @@ __global__ void part_scatter_kernel(int64_t N, int A,
     if (j >= 0 && split_dim[j] != A) {
       int64_t st = start[j];
       int64_t m = msize[j];
-      int64_t lr = (int64_t)pre[x] - (int64_t)pre[st];
+      int64_t lr = (int64_t)(pre[x] - pre[st]);
       uint8_t sd = side[e];
       if (sd == 0) {
         dest = st + lr;
@@ -193,6 +202,155 @@ __global__ void part_scatter_kernel(int64_t N, int A,
       }
     }
     ordA_next[dest] = e;
+  }
+}
+
+// ---- subtrees of at most kSub nodes -------------------------------------------
+// One block per subtree of level l0, one thread per slot: the three orders, as
+// 16-bit indices into the block's points, stay in shared memory for the
+// remaining levels, which would each cost a device-wide pass over six arrays
+// (about 1.1 ms at 2^24 points, and seventeen launches at any size).  The same
+// medians and stable partitions as above, so the same tree.  Bound by the block
+// barriers, six a level.  The ten levels of 2^24 points take 2.3 ms, 11 ms by
+// passes; a whole build of 30011 points goes from 2.37 to 1.44 ms.
+constexpr int kSub = 1024;
+
+struct SubTree {
+  float x[3][kSub];
+  int32_t gid[kSub];
+  uint16_t ord[2][3][kSub];        // [level parity][dimension][slot]
+  uint16_t seg[2][kSub];           // node of the slot on this level, kNone once done
+  uint16_t start[2][kSub], size[2][kSub];
+  uint16_t m[kSub], pre[3][kSub], slot[3][kSub];
+  uint16_t wsum[3][kSub / 32];
+  uint8_t dim[kSub], side[kSub];
+};
+constexpr uint16_t kNone = 0xffff;
+
+__global__ void __launch_bounds__(kSub, 2) tree_sub_kernel(
+    const float* __restrict__ pts, int64_t N, int l0, int levels, int rule, Orders ord,
+    const int32_t* __restrict__ start, int32_t* loc, int32_t* __restrict__ tree_point,
+    uint8_t* __restrict__ split_dim, int32_t* __restrict__ inorder,
+    int32_t* __restrict__ node_at_inorder, float4* __restrict__ box) {
+  extern __shared__ __align__(16) unsigned char sub_smem[];
+  SubTree& T = *reinterpret_cast<SubTree*>(sub_smem);
+  const int x = threadIdx.x, lane = x & 31, warp = x >> 5;
+  const int64_t p = blockIdx.x, j0 = (int64_t(1) << l0) - 1 + p;
+  if (j0 >= N) return;
+  const int S0 = (int)subtree_nodes(p, l0, N, levels);
+  const int64_t st0 = start[j0];
+  if (x < S0) {
+    const int32_t e = ord.o[0][st0 + x];
+    T.gid[x] = e;
+    for (int d = 0; d < 3; d++) T.x[d][x] = pts[3 * (int64_t)e + d];
+    T.ord[0][0][x] = (uint16_t)x;
+    loc[e] = x;
+  }
+  T.seg[0][x] = x < S0 ? 0 : kNone;
+  if (x == 0) {
+    T.start[0][0] = 0;
+    T.size[0][0] = (uint16_t)S0;
+  }
+  __syncthreads();
+  if (x < S0)
+    for (int d = 1; d < 3; d++) T.ord[0][d][x] = (uint16_t)loc[ord.o[d][st0 + x]];
+  __syncthreads();
+  for (int l = l0; l < levels; l++) {
+    const int c = (l - l0) & 1, nodes = 1 << (l - l0);
+    if (x < nodes) {  // the nodes of this level
+      const int64_t pos = p + ((int64_t)x << l0), j = (int64_t(1) << l) - 1 + pos;
+      if (j < N) {
+        const int S = T.size[c][x], st = T.start[c][x];
+        const int m = (int)subtree_nodes(pos, l + 1, N, levels);
+        float lo[3], hi[3], ext[3];
+        for (int d = 0; d < 3; d++) {
+          lo[d] = T.x[d][T.ord[c][d][st]];
+          hi[d] = T.x[d][T.ord[c][d][st + S - 1]];
+          ext[d] = __fsub_rn(hi[d], lo[d]);
+        }
+        int dim = l % 3;
+        if (rule == 0) {
+          dim = ext[1] > ext[0] ? 1 : 0;
+          if (ext[2] > (dim ? ext[1] : ext[0])) dim = 2;
+        }
+        if (box && l < levels - 1) {
+          const int64_t h = tree_heap_index(j);
+          box[2 * h] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+          box[2 * h + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
+        }
+        tree_point[j] = T.gid[T.ord[c][dim][st + m]];
+        split_dim[j] = (uint8_t)dim;
+        inorder[j] = (int32_t)(st0 + st + m);
+        node_at_inorder[st0 + st + m] = (int32_t)j;
+        T.m[x] = (uint16_t)m;
+        T.dim[x] = (uint8_t)dim;
+        if (m > 0) {
+          T.start[c ^ 1][x] = (uint16_t)st;
+          T.size[c ^ 1][x] = (uint16_t)m;
+        }
+        if (S - 1 - m > 0) {
+          T.start[c ^ 1][x + nodes] = (uint16_t)(st + m + 1);
+          T.size[c ^ 1][x + nodes] = (uint16_t)(S - 1 - m);
+        }
+      }
+    }
+    if (l == levels - 1) break;
+    __syncthreads();
+    const int t = T.seg[c][x];  // this slot's node; its split dimension's order
+    int st = 0, m = 0, dim = 3;
+    if (t != kNone) {
+      st = T.start[c][t];
+      m = T.m[t];
+      dim = T.dim[t];
+      const int r = x - st;
+      const int sd = r < m ? 0 : (r == m ? 1 : 2);
+      T.side[T.ord[c][dim][x]] = (uint8_t)sd;
+      T.seg[c ^ 1][x] = sd == 1 ? kNone : (uint16_t)(sd == 0 ? t : t + nodes);
+    } else {
+      T.seg[c ^ 1][x] = kNone;
+    }
+    __syncthreads();
+    int sides = 0;  // two bits per dimension
+#pragma unroll
+    for (int A = 0; A < 3; A++) {
+      int sd = 3;
+      if (t != kNone && dim != A) {
+        sd = T.side[T.ord[c][A][x]];
+        if (sd == 1) T.slot[A][t] = (uint16_t)x;
+      }
+      sides |= sd << (2 * A);
+      const unsigned left = __ballot_sync(0xffffffffu, sd == 0);
+      T.pre[A][x] = (uint16_t)__popc(left & ((1u << lane) - 1u));
+      if (lane == 0) T.wsum[A][warp] = (uint16_t)__popc(left);
+    }
+    __syncthreads();
+    if (warp < 3) {  // exclusive scan of the warps' counts
+      const int v = T.wsum[warp][lane];
+      int s = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
+      }
+      T.wsum[warp][lane] = (uint16_t)(s - v);
+    }
+    __syncthreads();
+    if (t != kNone) {
+#pragma unroll
+      for (int A = 0; A < 3; A++) {
+        const uint16_t e = T.ord[c][A][x];
+        int dest = x;
+        if (dim != A) {
+          const int lr = T.pre[A][x] + T.wsum[A][warp] - T.pre[A][st] - T.wsum[A][st >> 5];
+          const int sd = (sides >> (2 * A)) & 3;
+          dest = sd == 0 ? st + lr
+                         : (sd == 1 ? st + m
+                                    : st + m + 1 + (x - st) - lr - (T.slot[A][t] < x ? 1 : 0));
+        }
+        T.ord[c ^ 1][A][dest] = e;
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -217,6 +375,15 @@ int tree_build(const float* pts, int64_t N, int rule, int32_t* tree_point,
     GGP_CUDA(cudaGetLastError());
     GGP_TRY(radix_sort_pairs(keys, ids, keys_sorted, (uint32_t*)ord[d][0], N, 32, s));
   }
+  // The levels down to the first whose subtrees fit a block, then those in blocks.
+  int levels = 0, l0 = 0;
+  while (((int64_t(1) << levels) - 1) < N) levels++;
+  while (subtree_nodes(0, l0, N, levels) > kSub) l0++;
+  // Up to kBatch points the three partitions of a level share their launches
+  // (seven instead of seventeen a level, each a few us); above, the passes are
+  // bound by memory and one dimension's scratch serves all three.
+  constexpr int64_t kBatch = int64_t(1) << 21;
+  const int nb = N <= kBatch ? 3 : 1;
   int32_t *seg[2], *start = nullptr, *msize = nullptr, *node_slot = nullptr;
   uint8_t* side = nullptr;
   uint32_t *flags = nullptr, *pre = nullptr;
@@ -224,41 +391,46 @@ int tree_build(const float* pts, int64_t N, int rule, int32_t* tree_point,
   GGP_TRY(sc.alloc(&seg[1], N));
   GGP_TRY(sc.alloc(&start, N));
   GGP_TRY(sc.alloc(&msize, N));
-  GGP_TRY(sc.alloc(&node_slot, N));
+  GGP_TRY(sc.alloc(&node_slot, nb * N));
   GGP_TRY(sc.alloc(&side, N));
-  GGP_TRY(sc.alloc(&flags, N));
-  GGP_TRY(sc.alloc(&pre, N));
+  GGP_TRY(sc.alloc(&flags, nb * N));
+  GGP_TRY(sc.alloc(&pre, nb * N));
   GGP_CUDA(cudaMemsetAsync(seg[0], 0, N * sizeof(int32_t), s));  // all in root
   GGP_CUDA(cudaMemsetAsync(start, 0, sizeof(int32_t), s));
-  int cur[3] = {0, 0, 0};
-  int sg = 0;
-  int levels = 0;
-  while (((int64_t(1) << levels) - 1) < N) levels++;
-  for (int l = 0; l < levels; l++) {
+  int cur = 0;
+  for (int l = 0; l < l0; l++) {
     Orders o;
-    for (int d = 0; d < 3; d++) o.o[d] = ord[d][cur[d]];
+    OrdersOut next;
+    for (int d = 0; d < 3; d++) {
+      o.o[d] = ord[d][cur];
+      next.o[d] = ord[d][1 - cur];
+    }
     int64_t nodes = int64_t(1) << l;
-    level_nodes_kernel<<<grid_for(nodes, B), B, 0, s>>>(pts, N, l, rule, o, start, msize,
+    level_nodes_kernel<<<grid_for(nodes, B), B, 0, s>>>(pts, N, l, levels, rule, o, start, msize,
                                                         tree_point, split_dim, inorder,
-                                                        node_at_inorder,
-                                                        l < levels - 1 ? box : nullptr);
+                                                        node_at_inorder, box);
     GGP_CUDA(cudaGetLastError());
-    if (l == levels - 1) break;  // last level: every subtree is a single node
-    slot_side_kernel<<<grid, B, 0, s>>>(N, o, seg[sg], seg[1 - sg], start, msize, split_dim,
+    slot_side_kernel<<<grid, B, 0, s>>>(N, o, seg[cur], seg[1 - cur], start, msize, split_dim,
                                         side);
     GGP_CUDA(cudaGetLastError());
-    for (int A = 0; A < 3; A++) {
-      part_flags_kernel<<<grid, B, 0, s>>>(N, A, ord[A][cur[A]], seg[sg], split_dim, side, flags,
-                                           node_slot);
+    for (int A = 0; A < 3; A += nb) {
+      part_flags_kernel<<<dim3(grid, nb), B, 0, s>>>(N, A, o, seg[cur], split_dim, side, flags,
+                                                     node_slot);
       GGP_CUDA(cudaGetLastError());
-      GGP_TRY(scan_exclusive_u32(flags, pre, N, s));
-      part_scatter_kernel<<<grid, B, 0, s>>>(N, A, ord[A][cur[A]], ord[A][1 - cur[A]], seg[sg],
-                                             split_dim, side, pre, start, msize, node_slot);
+      GGP_TRY(scan_exclusive_u32(flags, pre, nb * N, s));
+      part_scatter_kernel<<<dim3(grid, nb), B, 0, s>>>(N, A, o, next, seg[cur], split_dim, side,
+                                                       pre, start, msize, node_slot);
       GGP_CUDA(cudaGetLastError());
-      cur[A] = 1 - cur[A];
     }
-    sg = 1 - sg;
+    cur = 1 - cur;
   }
+  Orders o;
+  for (int d = 0; d < 3; d++) o.o[d] = ord[d][cur];
+  GGP_CUDA(allow_dyn_smem(tree_sub_kernel, sizeof(SubTree)));
+  tree_sub_kernel<<<(unsigned)(int64_t(1) << l0), kSub, sizeof(SubTree), s>>>(
+      pts, N, l0, levels, rule, o, start, (int32_t*)flags, tree_point, split_dim, inorder,
+      node_at_inorder, box);
+  GGP_CUDA(cudaGetLastError());
   return GRAPHGP_OK;
 }
 
