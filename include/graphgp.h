@@ -227,8 +227,8 @@ int graphgp_nll_noalloc(graphgp_graph_t g, graphgp_factor_t f, const float* v_d,
  * graphgp_factor), so no graphgp_factor_t is needed and the device holds the
  * graph alone (about k + 4 words per point instead of 2k + 5).  For kernel
  * parameters that change at every step.  Requires k <= 32, else
- * GRAPHGP_ERR_INVALID (k <= 16: one thread per point; 16 < k <= 32: one warp
- * per point).  Results are bit-identical to graphgp_factor followed by the
+ * GRAPHGP_ERR_INVALID (k <= 16: two lanes per point; 16 < k <= 32: eight
+ * lanes per point).  Results are bit-identical to graphgp_factor followed by the
  * stored-factor sweep (the factor and the dot products run in the same
  * order); the log-determinant equals graphgp_logdet up to the order of its
  * FP64 partial sums.
@@ -253,8 +253,8 @@ int graphgp_nll_fused(graphgp_graph_t g, const graphgp_kernel* kern, const float
  * dNLL/d(lengthscale, sigma2, nugget) -- what graphgp_factor + graphgp_nll +
  * graphgp_nll_backward return, with one computation of every row's
  * conditional instead of two.  The form for kernel parameters that change at
- * every step (a fit).  k <= 32 (one thread per point for k <= 16, one warp
- * per point above); each call allocates stream-ordered scratch for the dense
+ * every step (a fit).  k <= 32 (two lanes per point for k <= 16, eight
+ * above); each call allocates stream-ordered scratch for the dense
  * block and the FP64 rescue list.  not_pd_d as for the other on-the-fly
  * calls.  vbar and thetabar agree with the stored-factor calls to rounding
  * (atomic sums). */

@@ -5,17 +5,17 @@
 // of 2k + 5 with stored weights); this is the form for kernel parameters that
 // change at every step.
 //
-// Two lanes own one point and run pair_factor (k <= 16; 16 < k
-// <= 32 in fused_group.cu) with the same FP64 rescue decision as the factor
-// kernel, so b and sigma are bit-identical to the stored factor's; the dot b . v_c then
+// Two lanes own one point and run pair_factor (k <= 16; 16 < k <= 32 in
+// fused_group.cu) with the same FP64 rescue decision as the factor kernel, so
+// b and sigma are bit-identical to the stored factor's; the dot b . v_c then
 // follows the stored sweeps' summation order (the row cut into gen_lanes(K)
 // slices, two alternating accumulators per slice, slices combined as their
 // xor-shuffle tree does), so the fused sweeps return the same bits as
 // factor + generate / whiten.
 //
 // generate: one cooperative launch over the depth levels with the level
-// barrier of the stored sweep; a thread computes the factor of its first
-// point of a level before waiting at the barrier, so the factor work of
+// barrier of the stored sweep; a block factors its first
+// points of a level before waiting at the barrier, so the factor work of
 // level l overlaps the end of level l - 1.  whiten: one grid-stride launch in
 // position order (no dependencies), optionally reducing xi.xi and
 // sum log sigma_i^2 in FP64.

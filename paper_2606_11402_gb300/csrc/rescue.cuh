@@ -132,9 +132,10 @@ __device__ __noinline__ void row_factor64(Row64<KMAX>& R, const float4* __restri
 // along and sigma^2 = K_ii - y.y summed in column order, and the backward
 // solve b = L^-T y.  A single thread needs k(k+1)/2 FP64 exponentials and
 // k^3/6 dependent FP64 multiply-adds for a row, at the low FP64 rate of this
-// GPU; the warp spreads both over its lanes.  Every path that rescues a row
-// with k <= 32 (factor, on-the-fly sweeps) uses this routine, so stored and
-// recomputed factors agree bit for bit.  All 32 lanes must call it with the
+// GPU; the warp spreads both over its lanes.  The on-the-fly paths with
+// k <= 32, which meet one row at a time, use this routine; listed rows go to
+// group_row_factor64, whose results are the same bits, so stored and recomputed
+// factors agree.  All 32 lanes must call it with the
 // same arguments; lane a receives b_a (0 for a >= k).
 struct WarpRow64 {
   double b;       // this lane's weight
