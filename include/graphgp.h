@@ -95,7 +95,14 @@ typedef struct {
   int32_t split_rule; /* k-d split dimension: 0 = widest bounding-box extent
                          (ties to the lowest dimension), 1 = level mod 3
                          (d = 3 only) */
-  int64_t max_spin;   /* bound on device spin iterations; 0 = default */
+  int64_t max_spin;   /* polls after which a device wait gives up
+                         (GRAPHGP_ERR_TIMEOUT); 0 = default 2 x 10^7.  A wait
+                         whose length follows from the sizes gets a fixed number
+                         more, so that no setting ends it early: the depths of
+                         the build 16 per point in flight, a panel of the dense
+                         block 2^20, generate without level barriers 1024 per
+                         level.  Level barriers get max_spin alone.  Graphs that
+                         are imported or loaded have the default. */
 } graphgp_build_opts;
 
 /* ---- graph construction (Sec. 2.2, Sec. 2.3 last paragraph) ------------
@@ -164,8 +171,9 @@ void graphgp_graph_destroy(graphgp_graph_t g);
  * block: L0 = chol(K_00) over positions 0..n0-1 and its inverse, sigma_i =
  * L0_ii (FP64 when flagged).  logdet = 2 sum_i log sigma_i is reduced in FP64
  * from the stored FP32 sigma.  Pivots below 1e-7 (kappa(0) + nugget) are
- * clamped to that value and counted (see graphgp_sync_status).  Allocates
- * stream-ordered scratch (a list of rows for the FP64 pass, FP64 work arrays
+ * clamped to that value and counted (see graphgp_sync_status).  The blocks
+ * that share the dense block wait for each other; a wait that gave up is
+ * reported by graphgp_sync_status.  Allocates stream-ordered scratch (a list of rows for the FP64 pass, FP64 work arrays
  * of 2 n0^2 doubles). */
 int graphgp_factor(graphgp_graph_t g, const graphgp_kernel* kern, void* stream,
                    graphgp_factor_t* out);

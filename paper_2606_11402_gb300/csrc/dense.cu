@@ -43,6 +43,11 @@ namespace {
 constexpr int kT = 32;            // tile edge
 constexpr int kDenseThreads = 256;
 constexpr int kDenseSplitMax = 320;  // largest n0 of the four-sum order
+// Polls that a wait for the other blocks' panel gets beside the graph's max_spin: a
+// panel is under 1 ms of work at any n0, a poll about 0.7 us.  A caller may bound
+// the waits of the sweeps tightly; the factor, which needs no such bound, has to
+// succeed all the same.
+constexpr int64_t kDensePolls = 1 << 20;
 
 struct DenseCheck {
   double logdet;           // sum log L0_ii^2 of the FP32 block
@@ -515,7 +520,7 @@ int dense_factor_kt(graphgp_graph_t g, graphgp_factor_t f, const KernF& kf, cuda
   d.chk = reinterpret_cast<DenseCheck*>(small);
   GGP_CUDA(cudaMemsetAsync(small, 0, nsmall * 4, s));
   GGP_CUDA(cudaMemsetAsync(&d.chk->min_piv, 0x7f, sizeof(int), s));  // 3.4e38
-  d.lb = LevelBarrier{small + sizeof(DenseCheck) / 4, g->err, g->max_spin};
+  d.lb = LevelBarrier{small + sizeof(DenseCheck) / 4, g->err, g->max_spin + kDensePolls};
   if (split)
     GGP_TRY((launch_dense<float, 4, KT>(d, s)));
   else

@@ -41,11 +41,14 @@ __global__ void canonicalise_kernel(const float* __restrict__ in, int d, float* 
 // needed.  In the bit-reversed order neighbours are spread over all earlier
 // points and few of a chunk's are in flight.  (The pass-per-launch form read
 // every row ~25 times per tree level with a host synchronisation each time:
-// 11.7 ms at 2^22 clustered points, k = 16.)  Waits are bounded: a block that
-// polls kDepthSpin times, or sees another's timeout, sets or finds
-// ERRBIT_TIMEOUT and leaves.
+// 11.7 ms at 2^22 clustered points, k = 16.)  Waits are bounded: a lane that has
+// polled limit times for its point, or sees another's timeout, sets or finds
+// ERRBIT_TIMEOUT and its block leaves.  The limit is the graph's max_spin
+// and kDepthPolls more for every point in flight: those may all be links of one
+// chain, a link takes a few round trips through L2, and a poll takes one.
 constexpr int kDepthChunk = 256;
-constexpr int64_t kDepthSpin = 20000000;  // polls before a wait gives up
+constexpr int kDepthBlocks = 8;  // per SM, at most
+constexpr int64_t kDepthPolls = 16;
 
 __device__ __forceinline__ int32_t ld_relaxed(const int32_t* p) {
   int32_t v;
@@ -60,7 +63,7 @@ __device__ __forceinline__ void st_relaxed(int32_t* p, int32_t v) {
 template <int U>
 __global__ void __launch_bounds__(kDepthChunk) depth_kernel(
     const int32_t* __restrict__ nbr_tree, int32_t* depth, int64_t N, int k, int64_t n0,
-    unsigned long long* __restrict__ ticket, int* __restrict__ dmax, uint32_t* err) {
+    unsigned long long* __restrict__ ticket, int* __restrict__ dmax, int64_t limit, uint32_t* err) {
   __shared__ unsigned long long s_chunk;
   int most = 0;
   bool dead = false;
@@ -101,7 +104,7 @@ __global__ void __launch_bounds__(kDepthChunk) depth_kernel(
           }
         } else if ((++spins & 255) == 0) {
           __nanosleep(100);
-          if (spins > kDepthSpin) atomicOr(err, ERRBIT_TIMEOUT);
+          if (spins > limit) atomicOr(err, ERRBIT_TIMEOUT);
           if (ld_relaxed((const int32_t*)err) & ERRBIT_TIMEOUT) {
             dead = true;
             open = false;
@@ -359,14 +362,15 @@ extern "C" int graphgp_build_graph(const float* points_d, int64_t N, int d, int 
     GGP_TRY(sc.alloc(&ticket, 2));
     GGP_CUDA(cudaMemsetAsync(ticket, 0, 16, s));
     if (N > n0) {
-      const unsigned grid = grid_for(N - n0, kDepthChunk, 8);
+      const unsigned grid = grid_for(N - n0, kDepthChunk, kDepthBlocks);
+      const int64_t limit = g->max_spin + kDepthPolls * grid * kDepthChunk;
       int* dmax = reinterpret_cast<int*>(ticket + 1);
       if (k >= 8)
         depth_kernel<8><<<grid, kDepthChunk, 0, s>>>(g->nbr_tree, g->depth_tree, N, k, n0,
-                                                     ticket, dmax, g->err);
+                                                     ticket, dmax, limit, g->err);
       else
         depth_kernel<4><<<grid, kDepthChunk, 0, s>>>(g->nbr_tree, g->depth_tree, N, k, n0,
-                                                     ticket, dmax, g->err);
+                                                     ticket, dmax, limit, g->err);
       GGP_CUDA(cudaGetLastError());
     }
     uint32_t e = 0;
