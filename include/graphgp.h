@@ -391,6 +391,11 @@ void graphgp_server_destroy(graphgp_server_t sv);
  * and recorded the timeout as designed (the context stays usable). */
 int graphgp_selftest_wait_timeout(int64_t max_spin, void* stream);
 
+/* The same for one kind of wait, on a value or count that never comes: which =
+ * 0 the level barrier (the call above), 1 the depths of the graph build, 2 the
+ * sweep without level barriers. */
+int graphgp_selftest_wait(int which, int64_t max_spin, void* stream);
+
 /* Writes the compute capability the library's device code was loaded for
  * (cudaFuncAttributes::binaryVersion of one of its kernels: major*10+minor,
  * 103 on GB300).  Not a paper operation.  Loads the module on the current

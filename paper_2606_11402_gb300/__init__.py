@@ -97,6 +97,7 @@ def load() -> ctypes.CDLL:
             "graphgp_nll_backward": [_P, _P, _P, ctypes.c_double, _P, _P, _P],
             "graphgp_nll_backward_points": [_P, _P, _P, ctypes.c_double, _P, _P],
             "graphgp_selftest_wait_timeout": [_I64, _P],
+            "graphgp_selftest_wait": [ctypes.c_int, _I64, _P],
             "graphgp_binary_version": [_P],
             "graphgp_factor_rows": [_P, _P, _I64, _I64, _P, _P],
             "graphgp_nll_rows": [_P, _P, _P, _P, _P],
@@ -421,6 +422,12 @@ def selftest_wait_timeout(max_spin: int = 20000, stream=None) -> int:
     """Runs the bounded-wait self-test; returns its status (ERR_TIMEOUT when the
     device waits gave up as designed)."""
     return load().graphgp_selftest_wait_timeout(int(max_spin), _stream(stream))
+
+
+def selftest_wait(which: int, max_spin: int = 20000, stream=None) -> int:
+    """The same for one kind of wait: 0 the level barrier, 1 the depths of the
+    graph build, 2 the sweep without level barriers."""
+    return load().graphgp_selftest_wait(int(which), int(max_spin), _stream(stream))
 
 
 def nll_noalloc(graph: Graph, fac: Factor, v: torch.Tensor, out: torch.Tensor,

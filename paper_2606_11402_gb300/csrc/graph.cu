@@ -258,6 +258,23 @@ int alloc_common(graphgp_graph_t g) {
 
 }  // namespace
 
+// The wait of the depth pass runs out: a point whose neighbour's depth is never
+// written.
+int depth_wait_selftest(int64_t limit, uint32_t* err, cudaStream_t s) {
+  Scratch sc(s);
+  int32_t* words = nullptr;  // depths of two points (not written), then the neighbour row
+  unsigned long long* ticket = nullptr;  // [0] next chunk, [1] the largest depth
+  GGP_TRY(sc.alloc(&words, 3));
+  GGP_TRY(sc.alloc(&ticket, 2));
+  GGP_CUDA(cudaMemsetAsync(words, 0xff, 2 * sizeof(int32_t), s));
+  GGP_CUDA(cudaMemsetAsync(words + 2, 0, sizeof(int32_t), s));
+  GGP_CUDA(cudaMemsetAsync(ticket, 0, 16, s));
+  depth_kernel<4><<<1, kDepthChunk, 0, s>>>(words + 2, words, 2, 1, 1, ticket,
+                                            reinterpret_cast<int*>(ticket + 1), limit, err);
+  GGP_CUDA(cudaGetLastError());
+  return GRAPHGP_OK;
+}
+
 // Level offsets on the device, the sweep barrier counters, and a check that
 // every neighbour lies in an earlier level.
 int graph_finish_device(graphgp_graph_t g, cudaStream_t s, bool have_keys) {

@@ -1,8 +1,9 @@
-// Self-test of the bounded device waits used by the level sweeps: every block
-// of a small cooperative launch waits at a level barrier whose count can never
-// reach the number of blocks (nothing arrives).  Each wait gives up after
-// max_spin polls, records ERRBIT_TIMEOUT and returns, so the launch ends and
-// the context stays usable; the host reads the error word.
+// Self-tests of the bounded device waits: a small launch waits for something that
+// never happens -- the level barrier of the sweeps for more arrivals than there
+// are blocks, the depth pass of the build (graph.cu) and the barrier-free sweep
+// (sweeps.cu) for a value that nobody writes.  Each wait gives up after max_spin
+// polls, records ERRBIT_TIMEOUT and returns, so the launch ends and the context
+// stays usable; the host reads the error word.
 #include "sweepsync.cuh"
 
 namespace ggp {
@@ -20,23 +21,34 @@ __global__ void barrier_timeout_kernel(LevelBarrier lb, uint32_t* reached) {
 
 using namespace ggp;
 
-extern "C" int graphgp_selftest_wait_timeout(int64_t max_spin, void* stream) {
-  if (max_spin < 1 || max_spin > ((int64_t)1 << 30)) return GRAPHGP_ERR_INVALID;
+extern "C" int graphgp_selftest_wait(int which, int64_t max_spin, void* stream) {
+  if (which < 0 || which > 2 || max_spin < 1 || max_spin > ((int64_t)1 << 30))
+    return GRAPHGP_ERR_INVALID;
   cudaStream_t s = (cudaStream_t)stream;
   Scratch sc(s);
   uint32_t* words = nullptr;  // [0] count, [1] error word, [2] reached
   GGP_TRY(sc.alloc(&words, 4));
   GGP_CUDA(cudaMemsetAsync(words, 0, 4 * sizeof(uint32_t), s));
-  LevelBarrier lb{words, words + 1, max_spin};
-  uint32_t* reached = words + 2;
-  void* args[] = {(void*)&lb, (void*)&reached};
-  GGP_CUDA(cudaLaunchCooperativeKernel((const void*)barrier_timeout_kernel, dim3(2), dim3(64), args,
-                                       0, s));
+  if (which == 0) {
+    LevelBarrier lb{words, words + 1, max_spin};
+    uint32_t* reached = words + 2;
+    void* args[] = {(void*)&lb, (void*)&reached};
+    GGP_CUDA(cudaLaunchCooperativeKernel((const void*)barrier_timeout_kernel, dim3(2), dim3(64),
+                                         args, 0, s));
+  } else if (which == 1) {
+    GGP_TRY(depth_wait_selftest(max_spin, words + 1, s));
+  } else {
+    GGP_TRY(flow_wait_selftest(max_spin, words + 1, s));
+  }
   uint32_t h[4] = {0, 0, 0, 0};
   GGP_CUDA(cudaMemcpyAsync(h, words, sizeof(h), cudaMemcpyDeviceToHost, s));
   GGP_CUDA(cudaStreamSynchronize(s));
   if (h[2] != 0) return GRAPHGP_ERR_INVALID;  // a wait passed without arrivals
   return (h[1] & ERRBIT_TIMEOUT) ? GRAPHGP_ERR_TIMEOUT : GRAPHGP_OK;
+}
+
+extern "C" int graphgp_selftest_wait_timeout(int64_t max_spin, void* stream) {
+  return graphgp_selftest_wait(0, max_spin, stream);
 }
 
 // Target of the device code actually loaded: binaryVersion of one of the

@@ -758,6 +758,32 @@ int launch_whiten(graphgp_graph_t g, graphgp_factor_t f, const float* v, float* 
 
 }  // namespace
 
+// The wait of the barrier-free sweep runs out: a point whose neighbour holds the
+// not-yet mark for good.
+int flow_wait_selftest(int64_t limit, uint32_t* err, cudaStream_t s) {
+  Scratch sc(s);
+  float* f = nullptr;    // v[2], then zeros: xi[2], sigma[2], and the weights at 8
+  int32_t* nbr = nullptr;
+  int64_t* off = nullptr;
+  GGP_TRY(sc.alloc(&f, 12));
+  GGP_TRY(sc.alloc(&nbr, 4));
+  GGP_TRY(sc.alloc(&off, 3));
+  const int64_t level_off[3] = {0, 1, 2};
+  GGP_CUDA(cudaMemsetAsync(f, 0, 12 * sizeof(float), s));
+  GGP_CUDA(cudaMemsetAsync(f, 0xff, 2 * sizeof(float), s));
+  GGP_CUDA(cudaMemsetAsync(nbr, 0, 4 * sizeof(int32_t), s));
+  GGP_CUDA(cudaMemcpyAsync(off, level_off, sizeof(level_off), cudaMemcpyHostToDevice, s));
+  const float *b = f + 8, *sigma = f + 4, *xi = f + 2;
+  int first = 1, levels = 2;
+  int64_t n0 = 1;
+  void* args[] = {(void*)&nbr, (void*)&b,     (void*)&sigma,  (void*)&xi, (void*)&f,    (void*)&off,
+                  (void*)&first, (void*)&levels, (void*)&n0, (void*)&limit, (void*)&err};
+  GGP_CUDA(cudaLaunchCooperativeKernel((const void*)generate_flow_kernel<4, 1, 2>, dim3(1),
+                                       dim3(kSweepThreads), args,
+                                       (2 * levels + 1) * sizeof(int32_t), s));
+  return GRAPHGP_OK;
+}
+
 int dense_matvec(const float* M, const float* x, float* y, int n0, double* sq, cudaStream_t s) {
   dense_lower_matvec_kernel<<<(n0 + 7) / 8, 256, 0, s>>>(M, x, y, n0, sq);
   GGP_CUDA(cudaGetLastError());
