@@ -114,6 +114,8 @@ typedef struct {
  * the depth of every point (d_i = 1 + max over c(i), dense block = 0), and
  * the depth-sorted graph order (ties by k-d tree in-order rank).
  * Synchronises `stream` (the host needs the number of depth levels).
+ * Allocates stream-ordered scratch of at most 70 bytes per point (above 2^21
+ * points; 24 more below).
  * Returns GRAPHGP_ERR_NAN for non-finite coordinates; -0.0 is read as +0.0. */
 int graphgp_build_graph(const float* points_d, int64_t N, int d, int k,
                         const graphgp_build_opts* opts, void* stream,

@@ -366,7 +366,7 @@ extern "C" int graphgp_build_graph(const float* points_d, int64_t N, int d, int 
     {
       Scratch bx(s);  // subtree boxes, only until the neighbours are found
       float4* box = nullptr;
-      GGP_TRY(bx.alloc(&box, (size_t)2 << (levels - 1)));
+      GGP_TRY(bx.alloc(&box, (size_t)1 << (levels - 1)));
       GGP_TRY(tree_build(g->pts_in, N, rule, g->tree_point, g->split_dim, g->inorder,
                          node_at_inorder, box, s));
       // preceding kNN

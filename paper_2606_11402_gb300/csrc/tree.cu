@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(kSub, 2) tree_sub_kernel(
           dim = ext[1] > ext[0] ? 1 : 0;
           if (ext[2] > (dim ? ext[1] : ext[0])) dim = 2;
         }
-        if (box && l < levels - 1) {
+        if (box && l < levels - 2) {
           const int64_t h = tree_heap_index(j);
           box[2 * h] = make_float4(lo[0], lo[1], lo[2], 0.0f);
           box[2 * h + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
@@ -361,20 +361,6 @@ int tree_build(const float* pts, int64_t N, int rule, int32_t* tree_point,
                float4* box, cudaStream_t s) {
   if (N <= 0) return GRAPHGP_OK;
   Scratch sc(s);
-  int32_t* ord[3][2];
-  uint32_t *keys = nullptr, *keys_sorted = nullptr, *ids = nullptr;
-  for (int d = 0; d < 3; d++)
-    for (int b = 0; b < 2; b++) GGP_TRY(sc.alloc(&ord[d][b], N));
-  GGP_TRY(sc.alloc(&keys, N));
-  GGP_TRY(sc.alloc(&keys_sorted, N));
-  GGP_TRY(sc.alloc(&ids, N));
-  const int B = 256;
-  unsigned grid = grid_for(N, B);
-  for (int d = 0; d < 3; d++) {
-    presort_keys_kernel<<<grid, B, 0, s>>>(pts, N, d, keys, ids);
-    GGP_CUDA(cudaGetLastError());
-    GGP_TRY(radix_sort_pairs(keys, ids, keys_sorted, (uint32_t*)ord[d][0], N, 32, s));
-  }
   // The levels down to the first whose subtrees fit a block, then those in blocks.
   int levels = 0, l0 = 0;
   while (((int64_t(1) << levels) - 1) < N) levels++;
@@ -384,17 +370,33 @@ int tree_build(const float* pts, int64_t N, int rule, int32_t* tree_point,
   // bound by memory and one dimension's scratch serves all three.
   constexpr int64_t kBatch = int64_t(1) << 21;
   const int nb = N <= kBatch ? 3 : 1;
-  int32_t *seg[2], *start = nullptr, *msize = nullptr, *node_slot = nullptr;
+  // Scratch, 45 bytes per point above kBatch: with the boxes (8 to 16) and
+  // node_at_inorder the build's peak stays below 70.  The presort's three arrays
+  // serve the partitions afterwards; start and msize hold the nodes of the levels
+  // done by passes and of the first done in blocks.
+  int32_t* ord[3][2];
+  uint32_t *keys = nullptr, *keys_sorted = nullptr, *ids = nullptr;
+  for (int d = 0; d < 3; d++)
+    for (int h = 0; h < 2; h++) GGP_TRY(sc.alloc(&ord[d][h], N));
+  GGP_TRY(sc.alloc(&keys, nb * N));
+  GGP_TRY(sc.alloc(&keys_sorted, nb * N));
+  GGP_TRY(sc.alloc(&ids, nb * N));
+  const int B = 256;
+  const unsigned grid = grid_for(N, B);
+  for (int d = 0; d < 3; d++) {
+    presort_keys_kernel<<<grid, B, 0, s>>>(pts, N, d, keys, ids);
+    GGP_CUDA(cudaGetLastError());
+    GGP_TRY(radix_sort_pairs(keys, ids, keys_sorted, (uint32_t*)ord[d][0], N, 32, s));
+  }
+  uint32_t *flags = keys, *pre = keys_sorted;
+  int32_t* node_slot = (int32_t*)ids;
+  int32_t *seg[2], *start = nullptr, *msize = nullptr;
   uint8_t* side = nullptr;
-  uint32_t *flags = nullptr, *pre = nullptr;
   GGP_TRY(sc.alloc(&seg[0], N));
   GGP_TRY(sc.alloc(&seg[1], N));
-  GGP_TRY(sc.alloc(&start, N));
-  GGP_TRY(sc.alloc(&msize, N));
-  GGP_TRY(sc.alloc(&node_slot, nb * N));
+  GGP_TRY(sc.alloc(&start, (size_t)2 << l0));
+  GGP_TRY(sc.alloc(&msize, (size_t)1 << l0));
   GGP_TRY(sc.alloc(&side, N));
-  GGP_TRY(sc.alloc(&flags, nb * N));
-  GGP_TRY(sc.alloc(&pre, nb * N));
   GGP_CUDA(cudaMemsetAsync(seg[0], 0, N * sizeof(int32_t), s));  // all in root
   GGP_CUDA(cudaMemsetAsync(start, 0, sizeof(int32_t), s));
   int cur = 0;
