@@ -249,22 +249,24 @@ __global__ void __launch_bounds__(small_threads(KP / LANES), 1) generate_small_k
 // generate against one block that gathers from L2 and a grid barrier for every
 // level above kTail: 46.4 -> 29.7 us (4096 points, k = 8), 66.9 -> 39.1 (4096,
 // k = 16), 88.4 -> 59.2 (10007, k = 16), 220 -> 188 (127001, k = 16).
-constexpr int kHeadThreads = 512;
+// Row slices of 28 entries (k = 25 .. 28, one lane per position) have half the
+// threads: two buffers of them need 112 registers.
+__host__ __device__ constexpr int head_threads(int hp) { return hp > 20 ? 256 : 512; }
 constexpr int64_t kHeadPoints = 49152;  // positions held (192 KB)
 constexpr int kHeadLevels = 4096;
 __host__ __device__ constexpr int head_depth(int hp) { return hp <= 4 ? 3 : (hp <= 8 ? 2 : 1); }
 
 template <int KP, int LANES>
-__global__ void __launch_bounds__(kHeadThreads, 1) generate_head_kernel(
+__global__ void __launch_bounds__(head_threads(KP / LANES), 1) generate_head_kernel(
     const int32_t* __restrict__ nbr, const float* __restrict__ b, const float* __restrict__ sigma,
     const float* __restrict__ xi, float* __restrict__ v, const int64_t* __restrict__ level_off,
     int l_end, int64_t n0) {
-  constexpr int HP = KP / LANES, PPB = kHeadThreads / LANES, D = head_depth(HP);
+  constexpr int HP = KP / LANES, NT = head_threads(HP), PPB = NT / LANES, D = head_depth(HP);
   extern __shared__ float s_v[];  // the field up to the last level's end, then the offsets
   const int32_t end = (int32_t)level_off[l_end];
   int32_t* s_lo = reinterpret_cast<int32_t*>(s_v + end);
-  for (int l = threadIdx.x; l <= l_end; l += kHeadThreads) s_lo[l] = (int32_t)level_off[l];
-  for (int i = threadIdx.x; i < (int)n0; i += kHeadThreads) s_v[i] = v[i];
+  for (int l = threadIdx.x; l <= l_end; l += NT) s_lo[l] = (int32_t)level_off[l];
+  for (int i = threadIdx.x; i < (int)n0; i += NT) s_v[i] = v[i];
   __syncthreads();
   const int h = threadIdx.x % LANES, slot = threadIdx.x / LANES;
   const uint64_t pol = l2_policy<0>();
@@ -342,6 +344,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1) generate_head_kernel(
 constexpr uint32_t kNotYet = 0xffffffffu;
 constexpr int kFlowMaxLevels = 4096;  // level table in shared memory
 constexpr int64_t kFlowEntries = 8 << 20;  // N times the padded row length
+constexpr int64_t kFlowLevel = 256 << 10;
 constexpr int64_t kFlowPolls = 1024;
 
 __device__ __forceinline__ uint32_t ld_flag(const float* p) {
@@ -661,19 +664,34 @@ int launch_generate(graphgp_graph_t g, graphgp_factor_t f, const float* xi, floa
   const int L = g->num_levels;
   if (L <= 1) return GRAPHGP_OK;
   constexpr int LANES = gen_lanes(KP), HP = KP / LANES, U = gen_steps(HP);
-  // The run of small levels that the sweep starts with (a level that one block
-  // covers in a few steps) goes to one block with its field in shared memory.
-  constexpr int64_t kSmall = 1024;
+  // The run of small levels that the sweep starts with goes to one block with its
+  // field in shared memory: levels of at most kSmall points and kSmallEntries row
+  // entries, which bound the block's loads.  generate with the line at 4 / 8 / 16 /
+  // 64 Ki entries, us: 30011 points, k = 16: 86 / 90 / 105 / 105, k = 32: 151 / 152 /
+  // 170 / 194, k = 64: 364 / 338 / 387 / 455; 127001, k = 16: 135 / 133 / 144 / 144,
+  // k = 48: 425 / 380 / 368 / 495; 10^6, k = 8: 132 / 129 / 130 / 130.  One lane per
+  // position takes more positions a step: 500,000, k = 12: 186 / 176 / 169 / 169.
+  // A cloud that the block can finish saves the other launch, so there a level may
+  // have 16 Ki entries and take kWholeSteps steps of the block: 10007 points,
+  // k = 1: 28.2 -> 24.0 (largest level 2346), k = 4: 34.1 -> 26.9, k = 48: 138 ->
+  // 129; with eight steps it loses (30011, k = 8: 54.8 -> 66.4).
+  constexpr int64_t kSmall = 1024, kSmallEntries = LANES == 1 ? 12288 : 8192;
+  constexpr int64_t kWholeSteps = 5;
   const std::vector<int64_t>& lo = g->level_off_h;
-  int a = 1;
-  while (a < L && a < kHeadLevels && lo[a + 1] - lo[a] <= kSmall && lo[a + 1] <= kHeadPoints) a++;
+  auto head_run = [&](int64_t most) {
+    int a = 1;
+    while (a < L && a < kHeadLevels && lo[a + 1] - lo[a] <= most && lo[a + 1] <= kHeadPoints) a++;
+    return a;
+  };
+  int a = head_run(std::min<int64_t>(16384 / KP, kWholeSteps * (head_threads(HP) / LANES)));
+  if (a < L) a = head_run(std::min(kSmall, kSmallEntries / KP));
   const int64_t* lod = g->level_off_d;
   int64_t n0 = g->n0;
   if (a > 1) {
     const size_t smem = (size_t)lo[a] * sizeof(float) + (a + 1) * sizeof(int32_t);
     auto kern = generate_head_kernel<KP, LANES>;
     GGP_CUDA(allow_dyn_smem(kern, smem));
-    kern<<<1, kHeadThreads, smem, s>>>(g->nbr, f->b, f->sigma, xi, v, lod, a, n0);
+    kern<<<1, head_threads(HP), smem, s>>>(g->nbr, f->b, f->sigma, xi, v, lod, a, n0);
     GGP_CUDA(cudaGetLastError());
   }
   if (a == L) return GRAPHGP_OK;
@@ -681,8 +699,10 @@ int launch_generate(graphgp_graph_t g, graphgp_factor_t f, const float* xi, floa
   // points, k = 16: 125 / 104; 127001, k = 7: 99 / 76; 10^6, k = 8: 168 / 143;
   // 500000, k = 16: 252 / 212; 262000, k = 32: 469 / 356; 130000, k = 64: 1058 /
   // 851.  Above, the values are no longer read soon after they are written: 10^6,
-  // k = 16: 286 / 294, k = 32: 603 / 1217; 2^24, k = 16: 902 / 1098.
-  const bool flow = g->N * KP <= kFlowEntries && L <= kFlowMaxLevels;
+  // k = 16: 286 / 294, k = 32: 603 / 1217; 2^24, k = 16: 902 / 1098.  And only with at
+  // most kFlowLevel entries a level on average, as what it saves is a barrier per
+  // level: 2 x 10^6, k = 1 (24 levels): 67 / 80, k = 4 (53 levels): 124 / 91.
+  const bool flow = g->N * KP <= std::min(kFlowEntries, kFlowLevel * L) && L <= kFlowMaxLevels;
   if (flow) return launch_generate_flow<KP>(g, f, xi, v, a, s);
   // the levels in between to the cooperative grid, the run of small ones at the
   // end (levels [z, L)) to one block
