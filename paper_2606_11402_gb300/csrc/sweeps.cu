@@ -741,8 +741,13 @@ int launch_whiten(graphgp_graph_t g, graphgp_factor_t f, const float* v, float* 
   // A tile is one block's work, so fewer than four per SM leave the chip idle or
   // its last wave nearly empty (tiles / in order, us; k = 16): 4096 points 74 / 16,
   // 10^6 136 / 60, 2^21 (3.4 tiles per SM) 143 / 104; 2^22 (6.7 per SM) 166 / 188,
-  // k = 8 92 / 98; 2^24 601 / 726: there the tile's gathers from L1 win.
-  const bool tiled = g->n_tiles >= 4 * (int64_t)num_sms();
+  // k = 8 92 / 98; 2^24 601 / 726: there the tile's gathers from L1 win.  k = 32: 2 x
+  // 10^6 182 / 148; k = 64: 1.5 x 10^6 314 / 315.  Rows of 20 or 28 entries on one lane
+  // are read in order at half the rate (U = 1, 16 bytes a lane apart), so they go to
+  // tiles earlier: k = 20: 750,000 (1.2 per SM) 70 / 64, 10^6 74 / 80; k = 28: 250,000
+  // (0.4 per SM) 58 / 46, 500,000 72 / 77, 10^6 103 / 134.
+  constexpr int64_t kQuarterTiles = gen_lanes(KP) > 1 || KP < 20 ? 16 : (KP < 28 ? 6 : 3);
+  const bool tiled = 4 * g->n_tiles >= kQuarterTiles * num_sms();
   if (tiled && g->tile_start && g->num_levels <= 8192) {
     size_t smem = (2 * (size_t)g->num_levels + 1) * sizeof(int32_t);
     GGP_CUDA(allow_dyn_smem(whiten_tiles_kernel<KP>, smem));
