@@ -438,10 +438,14 @@ __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) factor_ba
 // g = K_cc^-1 bbar by two triangular solves in shared memory.  Lane a + 32 s
 // takes row a + 32 s of Kbar against dK/dtheta (FP32 per row, FP64 across
 // rows); rows needing the FP64 rescue go to factor_backward_rescue_kernel.
+// Shared memory holds three blocks per SM, so the registers are set for three:
+// left to itself the compiler takes 64 and shortens the unrolled loops (400,000
+// rows, NLL gradient, k = 64: 52.6 ms with squared exponential, 56.3 Matern-3/2;
+// 43.1 and 45.0 with three blocks).
 template <int KT>
-__global__ void __launch_bounds__(128) factor_backward_wide_kernel(
+__global__ void __launch_bounds__(128, 3) factor_backward_wide_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int kp,
-    int64_t n0, KernF kf, int mode, const float* __restrict__ coef, float beta,
+    int64_t n0, KernF kf, double unit, int mode, const float* __restrict__ coef, float beta,
     const float* __restrict__ v, const float* __restrict__ xi, float* __restrict__ xibar_out,
     double* __restrict__ thetabar, int64_t* __restrict__ rescue_rows,
     unsigned long long* __restrict__ rescue_count) {
