@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) generate_
   using OL = OctLayout<K>;
   __shared__ int s_flag;
   extern __shared__ __align__(16) float psm[];
-  const int lane = threadIdx.x & 31, r = lane & 7, first = (threadIdx.x >> 5) * 4;
+  const int lane = threadIdx.x & 31, r = lane & 7, warp = threadIdx.x >> 5, first = warp * 4;
   float* S = psm + (threadIdx.x >> 3) * OL::kStride;
   const uint64_t pol_v = l2_evict_last();
   unsigned long long clamped = 0;
@@ -81,7 +81,9 @@ __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) generate_
     const int64_t steps = (hi - b0 + OL::kPoints - 1) / OL::kPoints;
     if (steps == 0 && l > 1 && lb.wait(l - 1, gridDim.x, &s_flag)) return;
     for (int64_t st = 0; st < steps; st++) {
-      const int64_t q = b0 + st * OL::kPoints + first + (lane >> 3);
+      // points dealt to the warps in turn: a warp recomputes its rows that need FP64
+      // one after the other
+      const int64_t q = b0 + st * OL::kPoints + (lane >> 3) * (kPairThreads / 32) + warp;
       const bool active = q < hi;
       const int64_t qq = active ? q : hi - 1;
       const int32_t* row = nbr + (qq - n0) * kp;
@@ -137,7 +139,14 @@ int generate_group_kt(graphgp_graph_t g, const KernF& kf, const float* xi, float
   static int max_grid_dev[kMaxDevices] = {};
   const int max_grid =
       coop_grid_cached(max_grid_dev, generate_fused_group_kernel<K, KT>, kPairThreads, smem);
-  const int64_t want = (g->max_level_size + OctLayout<K>::kPoints - 1) / OctLayout<K>::kPoints;
+  // Blocks for the largest level.  Where rows in FP64 are to be expected (no nugget,
+  // or all of them asked for) one point per warp: the FP64 unit of an SM does two
+  // lanes a clock, so what counts is the number of SMs.  Otherwise full blocks: more
+  // of them only cost the barrier (30,011 points, k = 32: 2.67 ms with full blocks,
+  // 2.73 / 2.99 / 3.65 with at least 152 / 304 / 456).
+  const bool fp64 = kf.nugd == 0.0 || kf.resc_T < 0.0f;
+  const int64_t per = fp64 ? kPairThreads / 32 : OctLayout<K>::kPoints;
+  const int64_t want = (g->max_level_size + per - 1) / per;
   const int grid = (int)std::min<int64_t>(max_grid, std::max<int64_t>(want, 1));
   GGP_CUDA(cudaMemsetAsync(g->level_bar, 0, g->num_levels * sizeof(uint32_t), s));
   LevelBarrier lb{g->level_bar, g->err, g->max_spin};
