@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) factor_ba
 template <int KT>
 __global__ void __launch_bounds__(128, 3) factor_backward_wide_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int kp,
-    int64_t n0, KernF kf, double unit, int mode, const float* __restrict__ coef, float beta,
+    int64_t n0, KernF kf, int mode, const float* __restrict__ coef, float beta,
     const float* __restrict__ v, const float* __restrict__ xi, float* __restrict__ xibar_out,
     double* __restrict__ thetabar, int64_t* __restrict__ rescue_rows,
     unsigned long long* __restrict__ rescue_count) {
