@@ -112,8 +112,10 @@ __device__ __forceinline__ double scaled(double t, double ljj) { return t / ljj;
 // accepted one in `pmin`) and D[j][r] and inv[j] (drcp of L_jj) are written; else they are read.
 // The row's entries are left in out[column][row] (DIAG: D itself) and, when lt
 // is given, in L0's transpose (lt: the row's entry of the tile's first column,
-// n0 apart; null for rows that do not exist).  `cols`: columns that exist.
-template <class T, int NP, bool DIAG>
+// n0 apart; null for rows that do not exist).  `cols`: columns that exist; fewer than
+// the tile's only on the last diagonal tile, which has a copy of this that stops
+// there (SHORT: a test per column makes every panel 3 % slower).
+template <class T, int NP, bool DIAG, bool SHORT = false>
 __device__ __noinline__ void tile_rows(const T* tile, T* D, T* inv, T* out, T* lt, int n0, int cols,
                                        T fl, unsigned& bad, T& pmin) {
   using F = DenseForm<T, NP>;
@@ -127,6 +129,11 @@ __device__ __noinline__ void tile_rows(const T* tile, T* D, T* inv, T* out, T* l
   }
 #pragma unroll
   for (int j = 0; j < kT; j++) {
+    if (SHORT && j >= cols) {
+      D[j * kT + r] = T(0);
+      if (r == j) inv[j] = T(1);
+      continue;
+    }
     T pl[F::planes];
 #pragma unroll
     for (int p = 0; p < NP; p++) pl[p] = a[p][j];
@@ -135,17 +142,15 @@ __device__ __noinline__ void tile_rows(const T* tile, T* D, T* inv, T* out, T* l
     T l;
     if (DIAG) {
       T piv = __shfl_sync(0xffffffffu, t, j);
-      const bool real = j < cols;
-      if (real && !(piv > fl)) {
+      if (!(piv > fl)) {
         piv = fl;
         bad++;
-      } else if (real) {
+      } else {
         pmin = piv < pmin ? piv : pmin;
       }
-      const T ljj = real ? droot(piv) : T(1);
+      const T ljj = droot(piv);
       const T iv = drcp(ljj);
       l = r > j ? scaled(t, iv) : (r == j ? ljj : T(0));
-      if (!real) l = T(0);
       D[j * kT + r] = l;
       if (r == j) inv[j] = iv;
       __syncwarp();
@@ -153,7 +158,7 @@ __device__ __noinline__ void tile_rows(const T* tile, T* D, T* inv, T* out, T* l
       l = scaled(t, inv[j]);
       out[j * kT + r] = l;
     }
-    if (lt && j < cols) lt[(int64_t)j * n0] = l;
+    if (lt) lt[(int64_t)j * n0] = l;
 #pragma unroll
     for (int c = j + 1; c < kT; c++) a[j % NP][c] = F::add(a[j % NP][c], l, D[j * kT + c]);
   }
@@ -367,9 +372,11 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_block_kernel(DenseArgs
       unsigned bad = 0;
       T pmin = k0;
       const bool own = a == J % px && b == J % py;  // writes it out
-      tile_rows<T, NP, true>(tile(J, J), D, inv, nullptr,
-                             own && lane < cols ? LT + (int64_t)J * kT * d.n0 + J * kT + lane : nullptr,
-                             d.n0, cols, fl, bad, pmin);
+      T* lt = own && lane < cols ? LT + (int64_t)J * kT * d.n0 + J * kT + lane : nullptr;
+      if (cols < kT)
+        tile_rows<T, NP, true, true>(tile(J, J), D, inv, nullptr, lt, d.n0, cols, fl, bad, pmin);
+      else
+        tile_rows<T, NP, true>(tile(J, J), D, inv, nullptr, lt, d.n0, cols, fl, bad, pmin);
       __syncwarp();
       if (own) {
         double ls = 0.0;
@@ -486,6 +493,11 @@ int launch_dense(DenseArgs d, cudaStream_t s) {
   const int grid = d.px == d.nb ? d.nb * (d.nb + 1) / 2 : d.px * d.py;
   const size_t smem = dense_smem<T, NP>(d.n0, (d.nb + d.px - 1) / d.px);
   GGP_CUDA(allow_dyn_smem(kern, smem));
+  if (grid == 1) {  // nothing to wait for: a plain launch, which costs less
+    kern<<<1, kDenseThreads, smem, s>>>(d);
+    GGP_CUDA(cudaGetLastError());
+    return GRAPHGP_OK;
+  }
   void* args[] = {(void*)&d};
   GGP_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(kDenseThreads), args,
                                        smem, s));
