@@ -398,6 +398,12 @@ int graphgp_selftest_wait_timeout(int64_t max_spin, void* stream);
  * sweep without level barriers. */
 int graphgp_selftest_wait(int which, int64_t max_spin, void* stream);
 
+/* Self-test of the square root and reciprocal that the FP32 factors use, on n
+ * arguments (device buffers of float[n]): root_d and inv_d by the scalar forms,
+ * pair_d the root by the packed form. */
+int graphgp_selftest_roots(const float* x_d, int64_t n, float* root_d, float* pair_d,
+                           float* inv_d, void* stream);
+
 /* Writes the compute capability the library's device code was loaded for
  * (cudaFuncAttributes::binaryVersion of one of its kernels: major*10+minor,
  * 103 on GB300).  Not a paper operation.  Loads the module on the current

@@ -98,6 +98,7 @@ def load() -> ctypes.CDLL:
             "graphgp_nll_backward_points": [_P, _P, _P, ctypes.c_double, _P, _P],
             "graphgp_selftest_wait_timeout": [_I64, _P],
             "graphgp_selftest_wait": [ctypes.c_int, _I64, _P],
+            "graphgp_selftest_roots": [_P, _I64, _P, _P, _P, _P],
             "graphgp_binary_version": [_P],
             "graphgp_factor_rows": [_P, _P, _I64, _I64, _P, _P],
             "graphgp_nll_rows": [_P, _P, _P, _P, _P],
@@ -428,6 +429,16 @@ def selftest_wait(which: int, max_spin: int = 20000, stream=None) -> int:
     """The same for one kind of wait: 0 the level barrier, 1 the depths of the
     graph build, 2 the sweep without level barriers."""
     return load().graphgp_selftest_wait(int(which), int(max_spin), _stream(stream))
+
+
+def selftest_roots(x: torch.Tensor, stream=None):
+    """(root, root by the packed form, reciprocal) of float32[n] as the FP32
+    factors evaluate them."""
+    out = [torch.empty_like(x) for _ in range(3)]
+    _check(load().graphgp_selftest_roots(_dev(x, torch.float32), x.numel(),
+                                         *(_dev(o, torch.float32) for o in out), _stream(stream)),
+           "selftest_roots")
+    return out
 
 
 def nll_noalloc(graph: Graph, fac: Factor, v: torch.Tensor, out: torch.Tensor,

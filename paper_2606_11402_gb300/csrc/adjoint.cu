@@ -181,7 +181,7 @@ __device__ void block_add3(double t0, double t1, double t2, double* out) {
 // theta_bar += sum_{a,b} Kbar[a][b] dK_ab/dtheta over the dense block.
 template <int KT>
 __global__ void dense_theta_kernel(const float* __restrict__ Kbar, const float4* __restrict__ xs,
-                                   int n0, KernF kf, double* __restrict__ thetabar) {
+                                   int n0, KernF kf, double unit, double* __restrict__ thetabar) {
   double tl = 0, ts = 0, tn = 0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)n0 * n0;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -196,7 +196,7 @@ __global__ void dense_theta_kernel(const float* __restrict__ Kbar, const float4*
       tl += (double)(kb * dkappa_dell_d2<KT>(kf, d2));
     }
   }
-  block_add3(tl, ts, tn, thetabar);
+  block_add3(tl * unit, ts, tn, thetabar);
 }
 
 // ---- adjoint sweeps by scatter ------------------------------------------------
@@ -393,7 +393,7 @@ int whiten_adjoint_scatter(graphgp_graph_t g, graphgp_factor_t f, const float* x
 template <int K, int KT>
 __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) factor_backward_oct_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int kp,
-    int64_t n0, KernF kf, int mode, const float* __restrict__ coef, float beta,
+    int64_t n0, KernF kf, double unit, int mode, const float* __restrict__ coef, float beta,
     const float* __restrict__ v, const float* __restrict__ xi, float* __restrict__ xibar_out,
     double* __restrict__ thetabar, int64_t* __restrict__ rescue_rows,
     unsigned long long* __restrict__ rescue_count) {
@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) factor_ba
         xibar_out[i] = f.sigma * ci;
     }
   }
-  block_add3(tl, ts, tn, thetabar);
+  block_add3(tl * unit, ts, tn, thetabar);
 }
 
 // The same per-row backward for 32 < k <= 64: one warp per point, the factor
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) factor_ba
 template <int KT>
 __global__ void __launch_bounds__(128, 3) factor_backward_wide_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int kp,
-    int64_t n0, KernF kf, int mode, const float* __restrict__ coef, float beta,
+    int64_t n0, KernF kf, double unit, int mode, const float* __restrict__ coef, float beta,
     const float* __restrict__ v, const float* __restrict__ xi, float* __restrict__ xibar_out,
     double* __restrict__ thetabar, int64_t* __restrict__ rescue_rows,
     unsigned long long* __restrict__ rescue_count) {
@@ -507,17 +507,17 @@ __global__ void __launch_bounds__(128, 3) factor_backward_wide_kernel(
     }
     __syncwarp();
   }
-  block_add3(tl, ts, tn, thetabar);
+  block_add3(tl * unit, ts, tn, thetabar);
 }
 
 // FP64 backward of the rows the per-row kernels handed over (rescue.cuh).
 template <int G, int KT>
 __global__ void __launch_bounds__(128) factor_backward_rescue_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int k, int kp, int64_t n0,
-    KernF kf, int mode, const float* __restrict__ coef, float beta, const float* __restrict__ v,
-    const float* __restrict__ xi, float* __restrict__ xibar_out, double* __restrict__ thetabar,
-    const int64_t* __restrict__ rows, const unsigned long long* __restrict__ count,
-    unsigned long long cap) {
+    KernF kf, double unit, int mode, const float* __restrict__ coef, float beta,
+    const float* __restrict__ v, const float* __restrict__ xi, float* __restrict__ xibar_out,
+    double* __restrict__ thetabar, const int64_t* __restrict__ rows,
+    const unsigned long long* __restrict__ count, unsigned long long cap) {
   double tl = 0.0, ts = 0.0, tn = 0.0;
   const int64_t n = (int64_t)(*count < cap ? *count : cap);
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n;
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(128) factor_backward_rescue_kernel(
     row_backward64<G, KT>(R, xs, row_ptr, k, xs[i], kf, v, al, sb, sg, tl, ts, tn);
     if (mode == 1) xibar_out[i] = sg * ci;
   }
-  block_add3(tl, ts, tn, thetabar);
+  block_add3(tl * unit, ts, tn, thetabar);
 }
 
 // The per-row backward for k <= 16: two lanes per point, the factor recomputed
@@ -541,10 +541,10 @@ __global__ void __launch_bounds__(128) factor_backward_rescue_kernel(
 template <int K, int KT>
 __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) factor_backward_pair_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int64_t n0,
-    KernF kf, int mode, const float* __restrict__ coef, float beta, const float* __restrict__ v,
-    const float* __restrict__ xi, float* __restrict__ xibar_out, double* __restrict__ thetabar,
-    int64_t* __restrict__ rescue_rows, unsigned long long* __restrict__ rescue_count,
-    unsigned long long rescue_cap) {
+    KernF kf, double unit, int mode, const float* __restrict__ coef, float beta,
+    const float* __restrict__ v, const float* __restrict__ xi, float* __restrict__ xibar_out,
+    double* __restrict__ thetabar, int64_t* __restrict__ rescue_rows,
+    unsigned long long* __restrict__ rescue_count, unsigned long long rescue_cap) {
   using PL = PairLayout<K>;
   extern __shared__ __align__(16) float psm[];
   const int lane = threadIdx.x & 31, r = lane & 1, first = (threadIdx.x >> 5) * 16;
@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) factor_b
     }
     __syncwarp();
   }
-  block_add3(tl, ts, tn, thetabar);
+  block_add3(tl * unit, ts, tn, thetabar);
 }
 
 // NLL value and gradient in one pass, the factors recomputed and never stored
@@ -610,9 +610,9 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) factor_b
 template <int K, int KT>
 __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) nll_grad_fused_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int64_t n0,
-    KernF kf, float nllbar, const float* __restrict__ v, float* vbar, float* __restrict__ xi_out,
-    float* __restrict__ xibar_out, double* __restrict__ thetabar, double* __restrict__ acc,
-    unsigned long long* __restrict__ not_pd, int64_t* __restrict__ rescue_rows,
+    KernF kf, double unit, float nllbar, const float* __restrict__ v, float* vbar,
+    float* __restrict__ xi_out, float* __restrict__ xibar_out, double* __restrict__ thetabar,
+    double* __restrict__ acc, unsigned long long* __restrict__ not_pd, int64_t* __restrict__ rescue_rows,
     unsigned long long* __restrict__ rescue_count, unsigned long long rescue_cap) {
   using PL = PairLayout<K>;
   extern __shared__ __align__(16) float psm[];
@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) nll_grad
     }
     __syncwarp();
   }
-  block_add3(tl, ts, tn, thetabar);
+  block_add3(tl * unit, ts, tn, thetabar);
   block_add_double(sq, acc);
   block_add_double(lacc.log_value(), acc + 1);
   unsigned long long c = clamped;
@@ -715,9 +715,9 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) nll_grad
 template <int K, int KP, int KT>
 __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) nll_grad_fused_oct_kernel(
     const float4* __restrict__ xs, const int32_t* __restrict__ nbr, int64_t N, int k, int64_t n0,
-    KernF kf, float nllbar, const float* __restrict__ v, float* vbar, float* __restrict__ xi_out,
-    float* __restrict__ xibar_out, double* __restrict__ thetabar, double* __restrict__ acc,
-    unsigned long long* __restrict__ not_pd, int64_t* __restrict__ rescue_rows,
+    KernF kf, double unit, float nllbar, const float* __restrict__ v, float* vbar,
+    float* __restrict__ xi_out, float* __restrict__ xibar_out, double* __restrict__ thetabar,
+    double* __restrict__ acc, unsigned long long* __restrict__ not_pd, int64_t* __restrict__ rescue_rows,
     unsigned long long* __restrict__ rescue_count) {
   using OL = OctLayout<K>;
   extern __shared__ __align__(16) float psm[];
@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) nll_grad_
     }
     __syncwarp();
   }
-  block_add3(tl, ts, tn, thetabar);
+  block_add3(tl * unit, ts, tn, thetabar);
   block_add_double(sq, acc);
   block_add_double(lacc.log_value(), acc + 1);
   unsigned long long c = clamped;
@@ -818,7 +818,8 @@ int launch_factor_backward_oct(graphgp_graph_t g, graphgp_factor_t f, int mode,
   if (npts <= 0) return GRAPHGP_OK;
   const unsigned grid = oct_grid<K>(npts);
   constexpr size_t smem = OctLayout<K>::kBytes;
-  KernF kf = make_kernf(f->kern);
+  const KernF kf = make_kernf(f->kern, g);
+  const double unit = graph_unit(g);
   Scratch sc(s);
   int64_t* rows = nullptr;
   unsigned long long* cnt = nullptr;
@@ -829,9 +830,9 @@ int launch_factor_backward_oct(graphgp_graph_t g, graphgp_factor_t f, int mode,
 #define GGP_FB(KT)                                                                          \
   GGP_CUDA(allow_dyn_smem(factor_backward_oct_kernel<K, KT>, smem));                        \
   factor_backward_oct_kernel<K, KT><<<grid, kPairThreads, smem, s>>>(                       \
-      g->xs, nbr, N, g->k, g->kp, n0v, kf, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt); \
+      g->xs, nbr, N, g->k, g->kp, n0v, kf, unit, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt); \
   factor_backward_rescue_kernel<K, KT><<<rgrid, 128, 0, s>>>(                               \
-      g->xs, nbr, g->k, g->kp, n0v, kf, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt, \
+      g->xs, nbr, g->k, g->kp, n0v, kf, unit, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt, \
       (unsigned long long)npts)
   switch (f->kern.type) {
     case GRAPHGP_MATERN12: GGP_FB(GRAPHGP_MATERN12); break;
@@ -854,7 +855,8 @@ int launch_factor_backward_pair(graphgp_graph_t g, graphgp_factor_t f, int mode,
   const int64_t npts = N - n0v;
   if (npts <= 0) return GRAPHGP_OK;
   const unsigned grid = pair_grid<K>(npts);
-  KernF kf = make_kernf(f->kern);
+  const KernF kf = make_kernf(f->kern, g);
+  const double unit = graph_unit(g);
   Scratch sc(s);
   const unsigned long long cap = (unsigned long long)std::min<int64_t>(npts, kBackwardRescueMax);
   int64_t* rows = nullptr;
@@ -867,10 +869,10 @@ int launch_factor_backward_pair(graphgp_graph_t g, graphgp_factor_t f, int mode,
 #define GGP_FBT(KT)                                                                             \
   GGP_CUDA(allow_dyn_smem(factor_backward_pair_kernel<K, KT>, smem));                         \
   factor_backward_pair_kernel<K, KT><<<grid, kPairThreads, smem, s>>>(                        \
-      g->xs, nbr, N, g->k, n0v, kf, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt, \
+      g->xs, nbr, N, g->k, n0v, kf, unit, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt, \
       cap);                                                                                     \
   factor_backward_rescue_kernel<K, KT><<<rgrid, 128, 0, s>>>(                                   \
-      g->xs, nbr, g->k, g->kp, n0v, kf, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt, cap)
+      g->xs, nbr, g->k, g->kp, n0v, kf, unit, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt, cap)
   switch (f->kern.type) {
     case GRAPHGP_MATERN12: GGP_FBT(GRAPHGP_MATERN12); break;
     case GRAPHGP_MATERN32: GGP_FBT(GRAPHGP_MATERN32); break;
@@ -890,7 +892,8 @@ int launch_nll_grad_fused(graphgp_graph_t g, const graphgp_kernel* kern, float n
   const int64_t npts = g->N - g->n0;
   if (npts <= 0) return GRAPHGP_OK;
   const unsigned grid = pair_grid<K>(npts);
-  const KernF kf = make_kernf(*kern);
+  const KernF kf = make_kernf(*kern, g);
+  const double unit = graph_unit(g);
   Scratch sc(s);
   const unsigned long long cap = (unsigned long long)std::min<int64_t>(npts, kBackwardRescueMax);
   int64_t* rows = nullptr;
@@ -903,10 +906,10 @@ int launch_nll_grad_fused(graphgp_graph_t g, const graphgp_kernel* kern, float n
 #define GGP_NGF(KT)                                                                              \
   GGP_CUDA(allow_dyn_smem(nll_grad_fused_kernel<K, KT>, smem));                                  \
   nll_grad_fused_kernel<K, KT><<<grid, kPairThreads, smem, s>>>(                                 \
-      g->xs, g->nbr, g->N, g->k, g->n0, kf, nllbar, v, vbar, xi_tmp, xibar_tmp, thetabar, acc,  \
+      g->xs, g->nbr, g->N, g->k, g->n0, kf, unit, nllbar, v, vbar, xi_tmp, xibar_tmp, thetabar, acc,  \
       not_pd, rows, cnt, cap);                                                                   \
   factor_backward_rescue_kernel<K, KT><<<rgrid, 128, 0, s>>>(                                    \
-      g->xs, g->nbr, g->k, g->kp, g->n0, kf, 0, xibar_tmp, nllbar, v, xi_tmp, nullptr, thetabar, \
+      g->xs, g->nbr, g->k, g->kp, g->n0, kf, unit, 0, xibar_tmp, nllbar, v, xi_tmp, nullptr, thetabar, \
       rows, cnt, cap)
   switch (kern->type) {
     case GRAPHGP_MATERN12: GGP_NGF(GRAPHGP_MATERN12); break;
@@ -928,7 +931,8 @@ int launch_nll_grad_fused_oct(graphgp_graph_t g, const graphgp_kernel* kern, flo
   if (npts <= 0) return GRAPHGP_OK;
   constexpr int K = KP <= 24 ? 24 : 32;
   const unsigned grid = oct_grid<K>(npts);
-  const KernF kf = make_kernf(*kern);
+  const KernF kf = make_kernf(*kern, g);
+  const double unit = graph_unit(g);
   Scratch sc(s);
   int64_t* rows = nullptr;
   unsigned long long* cnt = nullptr;
@@ -940,10 +944,10 @@ int launch_nll_grad_fused_oct(graphgp_graph_t g, const graphgp_kernel* kern, flo
 #define GGP_NGG(KT)                                                                              \
   GGP_CUDA(allow_dyn_smem(nll_grad_fused_oct_kernel<K, KP, KT>, smem));                          \
   nll_grad_fused_oct_kernel<K, KP, KT><<<grid, kPairThreads, smem, s>>>(                         \
-      g->xs, g->nbr, g->N, g->k, g->n0, kf, nllbar, v, vbar, xi_tmp, xibar_tmp, thetabar, acc,  \
+      g->xs, g->nbr, g->N, g->k, g->n0, kf, unit, nllbar, v, vbar, xi_tmp, xibar_tmp, thetabar, acc,  \
       not_pd, rows, cnt);                                                                        \
   factor_backward_rescue_kernel<K, KT><<<rgrid, 128, 0, s>>>(                                   \
-      g->xs, g->nbr, g->k, g->kp, g->n0, kf, 0, xibar_tmp, nllbar, v, xi_tmp, nullptr, thetabar, \
+      g->xs, g->nbr, g->k, g->kp, g->n0, kf, unit, 0, xibar_tmp, nllbar, v, xi_tmp, nullptr, thetabar, \
       rows, cnt, (unsigned long long)npts)
   switch (kern->type) {
     case GRAPHGP_MATERN12: GGP_NGG(GRAPHGP_MATERN12); break;
@@ -969,7 +973,8 @@ int launch_factor_backward_wide(graphgp_graph_t g, graphgp_factor_t f, int mode,
   constexpr int kWarps = 4;
   const size_t smem = kWarps * sizeof(WideWarp);
   const unsigned grid = grid_for((npts + kWarps - 1) / kWarps * 128, 128, 4);
-  KernF kf = make_kernf(f->kern);
+  const KernF kf = make_kernf(f->kern, g);
+  const double unit = graph_unit(g);
   Scratch sc(s);
   int64_t* rows = nullptr;
   unsigned long long* cnt = nullptr;
@@ -981,10 +986,10 @@ int launch_factor_backward_wide(graphgp_graph_t g, graphgp_factor_t f, int mode,
   GGP_CUDA(cudaFuncSetAttribute(factor_backward_wide_kernel<KT>,                               \
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));      \
   factor_backward_wide_kernel<KT><<<grid, 32 * kWarps, smem, s>>>(                             \
-      g->xs, nbr, N, g->k, g->kp, n0v, kf, mode, coef, beta, v, xi, xibar, thetabar,   \
+      g->xs, nbr, N, g->k, g->kp, n0v, kf, unit, mode, coef, beta, v, xi, xibar, thetabar,   \
       rows, cnt);                                                                              \
   factor_backward_rescue_kernel<kWideK, KT><<<rgrid, 128, 0, s>>>(                             \
-      g->xs, nbr, g->k, g->kp, n0v, kf, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt,  \
+      g->xs, nbr, g->k, g->kp, n0v, kf, unit, mode, coef, beta, v, xi, xibar, thetabar, rows, cnt,  \
       (unsigned long long)npts)
   switch (f->kern.type) {
     case GRAPHGP_MATERN12: GGP_FBW(GRAPHGP_MATERN12); break;
@@ -1055,12 +1060,13 @@ int dense_backward(graphgp_graph_t g, graphgp_factor_t f, const float* u0, const
   GGP_TRY(sc.alloc(&Lb, nn));
   GGP_TRY(dense_kbar(g, f, u0, xi0, sgn, ldbar, Lb, s));
   unsigned grid = grid_for(nn, 256);
-  KernF kf = make_kernf(f->kern);
+  const KernF kf = make_kernf(f->kern, g);
+  const double unit = graph_unit(g);
   switch (f->kern.type) {
-    case GRAPHGP_MATERN12: dense_theta_kernel<GRAPHGP_MATERN12><<<grid, 256, 0, s>>>(Lb, g->xs, n0, kf, thetabar); break;
-    case GRAPHGP_MATERN32: dense_theta_kernel<GRAPHGP_MATERN32><<<grid, 256, 0, s>>>(Lb, g->xs, n0, kf, thetabar); break;
-    case GRAPHGP_MATERN52: dense_theta_kernel<GRAPHGP_MATERN52><<<grid, 256, 0, s>>>(Lb, g->xs, n0, kf, thetabar); break;
-    default: dense_theta_kernel<GRAPHGP_SQEXP><<<grid, 256, 0, s>>>(Lb, g->xs, n0, kf, thetabar); break;
+    case GRAPHGP_MATERN12: dense_theta_kernel<GRAPHGP_MATERN12><<<grid, 256, 0, s>>>(Lb, g->xs, n0, kf, unit, thetabar); break;
+    case GRAPHGP_MATERN32: dense_theta_kernel<GRAPHGP_MATERN32><<<grid, 256, 0, s>>>(Lb, g->xs, n0, kf, unit, thetabar); break;
+    case GRAPHGP_MATERN52: dense_theta_kernel<GRAPHGP_MATERN52><<<grid, 256, 0, s>>>(Lb, g->xs, n0, kf, unit, thetabar); break;
+    default: dense_theta_kernel<GRAPHGP_SQEXP><<<grid, 256, 0, s>>>(Lb, g->xs, n0, kf, unit, thetabar); break;
   }
   GGP_CUDA(cudaGetLastError());
   return GRAPHGP_OK;

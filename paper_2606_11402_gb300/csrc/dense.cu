@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_block_kernel(DenseArgs
   __syncthreads();
   d.lb.arrive(0);
   const T k0 = sizeof(T) == 4 ? T(d.kf.s2 + d.kf.nug) : T(d.kf.s2d + d.kf.nugd);
-  const T fl = sizeof(T) == 4 ? T(kPdFloor * (float)k0) : T(kPdFloor64 * k0);
+  const T fl = sizeof(T) == 4 ? T(fmaxf(kPdFloor * (float)k0, kPivotMin)) : T(kPdFloor64 * k0);
   for (int J = 0; J < nb; J++) {
     if (d.lb.wait(J, gridDim.x, &s_flag)) return;
     const int cols = min(kT, d.n0 - J * kT);

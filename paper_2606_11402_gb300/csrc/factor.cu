@@ -445,7 +445,7 @@ static int factor_impl(graphgp_graph_t g, const graphgp_kernel* kern, int64_t p0
     GGP_TRY(f->mem.alloc(&f->not_pd, 1));
     GGP_CUDA(cudaMemsetAsync(f->logdet, 0, 8, s));
     GGP_CUDA(cudaMemsetAsync(f->not_pd, 0, 8, s));
-    KernF kf = make_kernf(*kern);
+    KernF kf = make_kernf(*kern, g);
     if (rows) {  // rows outside the range stay zero
       GGP_CUDA(cudaMemsetAsync(f->b, 0, (g->N - g->n0) * g->kp * sizeof(float), s));
       GGP_CUDA(cudaMemsetAsync(f->sigma, 0, g->N * sizeof(float), s));

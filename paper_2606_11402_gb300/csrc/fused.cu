@@ -150,7 +150,7 @@ int dense_into(graphgp_graph_t g, const graphgp_kernel* kern, Scratch& sc, doubl
   GGP_TRY(sc.alloc(&f.sigma, g->n0));
   f.logdet = logdet;
   f.not_pd = not_pd;
-  return dense_factor(g, &f, make_kernf(*kern), kern->type, s);
+  return dense_factor(g, &f, make_kernf(*kern, g), kern->type, s);
 }
 
 namespace {
@@ -228,7 +228,7 @@ int whiten_fused(graphgp_graph_t g, const graphgp_kernel* kern, const float* v, 
   int rc = dense_into(g, kern, sc, logdet, not_pd, f, s);
   if (rc == GRAPHGP_OK) rc = dense_matvec(f.L0inv, v, xi, g->n0, sq, s);
   if (rc == GRAPHGP_OK) {
-    const KernF kf = make_kernf(*kern);
+    const KernF kf = make_kernf(*kern, g);
     if (g->kp > 16) return whiten_fused_group(g, kern->type, kf, v, xi, sq, logdet, not_pd, s);
 #define GGP_CALL(K) rc = launch_whiten_fused<K>(g, kern->type, kf, v, xi, sq, logdet, not_pd, s)
     GGP_FUSED_DISPATCH(GGP_CALL)
@@ -264,7 +264,7 @@ extern "C" int graphgp_generate_fused(graphgp_graph_t g, const graphgp_kernel* k
   int rc = dense_into(g, kern, sc, ld, bad, f, s);
   if (rc == GRAPHGP_OK) rc = dense_matvec(f.L0, xi_d, v_d, g->n0, nullptr, s);
   if (rc == GRAPHGP_OK) {
-    const KernF kf = make_kernf(*kern);
+    const KernF kf = make_kernf(*kern, g);
     if (g->kp > 16) return generate_fused_group(g, kern->type, kf, xi_d, v_d, bad, s);
 #define GGP_CALL(K) rc = launch_generate_fused<K>(g, kern->type, kf, xi_d, v_d, bad, s)
     GGP_FUSED_DISPATCH(GGP_CALL)

@@ -17,18 +17,31 @@ namespace {
 // coordinates: distances are unchanged (exact zero terms), and the widest-
 // extent split never picks a zero-extent dimension while a real one has a
 // positive extent (all extents zero: lowest dimension, as in d dimensions).
+// bad[0] counts non-finite coordinates, bad[1] those below kCloseCoord but not zero.
 __global__ void canonicalise_kernel(const float* __restrict__ in, int d, float* __restrict__ out,
                                     int64_t n, unsigned long long* __restrict__ bad) {
-  unsigned long long local = 0;
+  unsigned long long local = 0, close = 0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * 3;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / 3;
     const int c = (int)(e - i * 3);
     float x = c < d ? in[i * d + c] : 0.0f;
     if (!isfinite(x)) local++;
+    if (x != 0.0f && fabsf(x) < kCloseCoord) close++;
     out[e] = (x == 0.0f) ? 0.0f : x;  // -0.0 becomes +0.0
   }
   if (local) atomicAdd(bad, local);
+  if (close) atomicAdd(bad + 1, close);
+}
+
+// Largest absolute value of finite x (its bits, which order as the values do).
+__global__ void largest_kernel(const float* __restrict__ x, int64_t n,
+                               unsigned* __restrict__ out) {
+  unsigned most = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    most = max(most, __float_as_uint(fabsf(x[i])));
+  atomicMax(out, most);
 }
 
 // Depth, d_j = 1 + max over c(j) of d_i (the fixed point of Sec. 2.3 in one
@@ -145,10 +158,16 @@ __global__ void depth_keys_kernel(const int32_t* __restrict__ node_at_inorder,
       if (hist[i]) atomicAdd(level_count + i, (unsigned long long)hist[i]);
 }
 
+// A point in the graph's unit, 2^unit_exp (exact).
+__device__ __forceinline__ float4 point_in_unit(const float* p, int unit_exp) {
+  if (unit_exp == 0) return make_float4(p[0], p[1], p[2], 0.0f);
+  return make_float4(ldexpf(p[0], unit_exp), ldexpf(p[1], unit_exp), ldexpf(p[2], unit_exp), 0.0f);
+}
+
 __global__ void positions_kernel(const uint32_t* __restrict__ tree_of_pos,
                                  const int32_t* __restrict__ tree_point,
                                  const int32_t* __restrict__ inorder,
-                                 const float* __restrict__ pts, int64_t N,
+                                 const float* __restrict__ pts, int64_t N, int unit_exp,
                                  int32_t* __restrict__ pos_of_tree, int32_t* __restrict__ order,
                                  float4* __restrict__ xs, int32_t* __restrict__ pos_key) {
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
@@ -158,7 +177,7 @@ __global__ void positions_kernel(const uint32_t* __restrict__ tree_of_pos,
     pos_key[p] = inorder[j];
     int64_t o = tree_point[j];
     order[p] = (int32_t)o;
-    xs[p] = make_float4(pts[3 * o], pts[3 * o + 1], pts[3 * o + 2], 0.0f);
+    xs[p] = point_in_unit(pts + 3 * o, unit_exp);
   }
 }
 
@@ -181,11 +200,11 @@ __global__ void relabel_kernel(const uint32_t* __restrict__ tree_of_pos,
 }
 
 __global__ void order_xs_kernel(const float* __restrict__ pts, const int32_t* __restrict__ order,
-                                int64_t N, float4* __restrict__ xs) {
+                                int64_t N, int unit_exp, float4* __restrict__ xs) {
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
        p += (int64_t)gridDim.x * blockDim.x) {
     int64_t o = order[p];
-    xs[p] = make_float4(pts[3 * o], pts[3 * o + 1], pts[3 * o + 2], 0.0f);
+    xs[p] = point_in_unit(pts + 3 * o, unit_exp);
   }
 }
 
@@ -343,15 +362,23 @@ extern "C" int graphgp_build_graph(const float* points_d, int64_t N, int d, int 
   rc = [&]() -> int {
     Scratch sc(s);
     unsigned long long* bad = nullptr;
-    GGP_TRY(sc.alloc(&bad, 1));
-    GGP_CUDA(cudaMemsetAsync(bad, 0, 8, s));
+    GGP_TRY(sc.alloc(&bad, 3));
+    GGP_CUDA(cudaMemsetAsync(bad, 0, 24, s));
     GGP_CUDA(cudaMemsetAsync(g->err, 0, 4, s));
     canonicalise_kernel<<<grid_for(N * 3, 256), 256, 0, s>>>(points_d, d, g->pts_in, N, bad);
     GGP_CUDA(cudaGetLastError());
-    unsigned long long nbad = 0;
-    GGP_CUDA(cudaMemcpyAsync(&nbad, bad, 8, cudaMemcpyDeviceToHost, s));
+    unsigned long long nbad[2] = {0, 0};
+    GGP_CUDA(cudaMemcpyAsync(nbad, bad, 16, cudaMemcpyDeviceToHost, s));
     GGP_CUDA(cudaStreamSynchronize(s));
-    if (nbad) return GRAPHGP_ERR_NAN;
+    if (nbad[0]) return GRAPHGP_ERR_NAN;
+    if (nbad[1]) {
+      float most = 0.0f;
+      largest_kernel<<<grid_for(N * 3, 256), 256, 0, s>>>(g->pts_in, N * 3, (unsigned*)(bad + 2));
+      GGP_CUDA(cudaGetLastError());
+      GGP_CUDA(cudaMemcpyAsync(&most, bad + 2, 4, cudaMemcpyDeviceToHost, s));
+      GGP_CUDA(cudaStreamSynchronize(s));
+      g->unit_exp = close_unit_exp(most);
+    }
     // tree
     GGP_TRY(g->mem.alloc(&g->tree_point, N));
     GGP_TRY(g->mem.alloc(&g->split_dim, N));
@@ -417,8 +444,8 @@ extern "C" int graphgp_build_graph(const float* points_d, int64_t N, int d, int 
     int32_t* pos_of_tree = nullptr;
     GGP_TRY(sc.alloc(&pos_of_tree, N));
     positions_kernel<<<grid_for(N, 256), 256, 0, s>>>(tree_of_pos, g->tree_point, g->inorder,
-                                                      g->pts_in, N, pos_of_tree, g->order, g->xs,
-                                                      (int32_t*)g->tmp_vec);
+                                                      g->pts_in, N, g->unit_exp, pos_of_tree, g->order,
+                                                      g->xs, (int32_t*)g->tmp_vec);
     GGP_CUDA(cudaGetLastError());
     if (N > n0) {
       relabel_kernel<<<grid_for((N - n0) * g->kp, 256), 256, 0, s>>>(
@@ -493,8 +520,14 @@ extern "C" int graphgp_graph_import(const float* points_h, int64_t N, int k, int
   if (rc < 0) return fail(rc);
   rc = [&]() -> int {
     std::vector<float> pts(points_h, points_h + N * 3);
-    for (auto& x : pts)
+    bool close = false;
+    float most = 0.0f;
+    for (auto& x : pts) {
       if (x == 0.0f) x = 0.0f;
+      close |= x != 0.0f && std::fabs(x) < kCloseCoord;
+      most = std::max(most, std::fabs(x));
+    }
+    if (close) g->unit_exp = close_unit_exp(most);
     std::vector<int32_t> nbrp((size_t)(N - n0) * g->kp, 0);
     for (int64_t r = 0; r < N - n0; r++)
       std::memcpy(&nbrp[r * g->kp], nbr_h + r * k, k * sizeof(int32_t));
@@ -503,7 +536,8 @@ extern "C" int graphgp_graph_import(const float* points_h, int64_t N, int k, int
     GGP_CUDA(cudaMemcpyAsync(g->order, order_h, N * 4, cudaMemcpyHostToDevice, s));
     if (N > n0)
       GGP_CUDA(cudaMemcpyAsync(g->nbr, nbrp.data(), nbrp.size() * 4, cudaMemcpyHostToDevice, s));
-    order_xs_kernel<<<grid_for(N, 256), 256, 0, s>>>(g->pts_in, g->order, N, g->xs);
+    order_xs_kernel<<<grid_for(N, 256), 256, 0, s>>>(g->pts_in, g->order, N, g->unit_exp,
+                                                     g->xs);
     GGP_CUDA(cudaGetLastError());
     GGP_CUDA(cudaStreamSynchronize(s));
     return GRAPHGP_OK;

@@ -249,7 +249,7 @@ __device__ __forceinline__ void oct_factor(OctFactor<K>& f, float* S, int r, int
   DF s2{f.varw, 0.0f};
   bool clamped = false;
   float max_ratio = 1.0f;
-  const float pfloor = kPdFloor * k0;
+  const float pfloor = fmaxf(kPdFloor * k0, kPivotMin);
 #pragma unroll
   for (int s = 0; s < R; s++) f.b[s] = 0.0f;
   static_for<0, K>([&](auto Jc) {

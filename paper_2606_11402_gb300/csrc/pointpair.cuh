@@ -375,7 +375,7 @@ __device__ __forceinline__ void pair_factor(PairFactor<K>& f, float* S, int r, i
   DF s2{f.varw, 0.0f};
   bool clamped = false;
   float max_ratio = 1.0f;
-  const float pfloor = kPdFloor * k0;
+  const float pfloor = fmaxf(kPdFloor * k0, kPivotMin);
   static_for<0, K>([&](auto Jc) {
     constexpr int j = decltype(Jc)::value;
     constexpr int sj = j / 2, rj = j % 2;

@@ -91,7 +91,7 @@ __device__ __forceinline__ WideFactor point_factor_wide(WideWarp& W, int k, cons
   __syncwarp();
   WideFactor r{0.0f, false, 1.0f, inc ? 2.0f * (e0i + nug) : k0, inc};
   DF s2{r.varw, 0.0f};
-  const float pfloor = kPdFloor * k0;
+  const float pfloor = fmaxf(kPdFloor * k0, kPivotMin);
   for (int j = 0; j < k; j++) {
     float piv = W.L[j * kWideLd + j];
     if (!(piv > pfloor)) {

@@ -202,16 +202,17 @@ __global__ void dense_position_kernel(const float* __restrict__ Kbar,
   }
 }
 
-// out[order[p]] = acc[p] (graph order -> input order), FP64 -> FP32.
+// out[order[p]] = unit acc[p] (graph order -> input order, the graph's unit -> the
+// points'), FP64 -> FP32.
 __global__ void scatter_points_kernel(const double* __restrict__ acc,
-                                      const int32_t* __restrict__ order, int64_t N,
+                                      const int32_t* __restrict__ order, int64_t N, double unit,
                                       float* __restrict__ out) {
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
        p += (int64_t)gridDim.x * blockDim.x) {
     const int64_t q = order[p];
-    out[3 * q] = (float)acc[3 * p];
-    out[3 * q + 1] = (float)acc[3 * p + 1];
-    out[3 * q + 2] = (float)acc[3 * p + 2];
+    out[3 * q] = (float)(unit * acc[3 * p]);
+    out[3 * q + 1] = (float)(unit * acc[3 * p + 1]);
+    out[3 * q + 2] = (float)(unit * acc[3 * p + 2]);
   }
 }
 
@@ -230,7 +231,7 @@ int launch_positions(graphgp_graph_t g, graphgp_factor_t f, const float* v, cons
                      float nllbar, double* acc, cudaStream_t s) {
   const int n0 = g->n0;
   const int64_t npts = g->N - n0;
-  const KernF kf = make_kernf(f->kern);
+  const KernF kf = make_kernf(f->kern, g);
   Scratch sc(s);
   // dense block
   float *u0 = nullptr, *Kbar = nullptr;
@@ -286,7 +287,8 @@ extern "C" int graphgp_nll_backward_points(graphgp_graph_t g, graphgp_factor_t f
     default: rc = launch_positions<GRAPHGP_SQEXP>(g, f, v_d, xi, (float)nllbar, acc, s); break;
   }
   if (rc < 0) return rc;
-  scatter_points_kernel<<<grid_for(g->N, 256), 256, 0, s>>>(acc, g->order, g->N, pbar_d);
+  scatter_points_kernel<<<grid_for(g->N, 256), 256, 0, s>>>(acc, g->order, g->N,
+                                                            graph_unit(g), pbar_d);
   GGP_CUDA(cudaGetLastError());
   return GRAPHGP_OK;
 }
