@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(kPairThreads, PairLayout<K>::kBlocks) nll_grad
       const WarpRow64 wr = warp_row_factor64<K, KT>(
           xs, row, k, xu, kf, reinterpret_cast<double*>(psm + first * PL::kStride));
       const float b = lane < k ? (float)wr.b : 0.0f, sg = (float)wr.sigma;
-      const float dot = warp_dot_stored_order<K, false>(b, row, v, pol_v);
+      const float dot = warp_dot_stored_order<K>(b, row, v, pol_v);
       const float xu0 = __shfl_sync(full, (ld_keep_f(v + iu, pol_v) - dot) / sg, 0);
       const float xbu = nllbar * xu0, wu = xbu / sg;
       if (lane < k && b != 0.0f) atomicAdd(vbar + row[lane], b * -wu);
@@ -771,7 +771,7 @@ __global__ void __launch_bounds__(kPairThreads, OctLayout<K>::kBlocks) nll_grad_
       const WarpRow64 wr = oct_row64<K, KT>(xs, ru, k, __ldg(xs + iu), kf,
                                          reinterpret_cast<double*>(psm + first * OL::kStride));
       const float b = lane < k ? (float)wr.b : 0.0f, sg = (float)wr.sigma;
-      const float dot = warp_dot_stored_order<KP, false>(b, ru, v, pol_v);
+      const float dot = warp_dot_stored_order<KP>(b, ru, v, pol_v);
       const float xu = __shfl_sync(full, (ld_keep_f(v + iu, pol_v) - dot) / sg, 0);
       const float xbu = nllbar * xu, wu = xbu / sg;
       if (lane < k && b != 0.0f) atomicAdd(vbar + ru[lane], b * -wu);

@@ -179,7 +179,7 @@ __host__ __device__ constexpr int gen_lanes(int kp) { return kp % 16 == 0 ? 4 : 
 // holds b_a (b_own);
 // lane h of the warp forms slice h from the shuffled weights and the row's
 // neighbour indices (padding entries included).  Valid on lane 0.
-template <int KP, bool LEVEL>
+template <int KP>
 __device__ __forceinline__ float warp_dot_stored_order(float b_own, const int32_t* row,
                                                        const float* v, uint64_t pol) {
   constexpr int LANES = gen_lanes(KP), HP = KP / LANES;
@@ -193,14 +193,8 @@ __device__ __forceinline__ float warp_dot_stored_order(float b_own, const int32_
     const float w1 = __shfl_sync(0xffffffffu, b_own, (e + 1) & 31);
     const float w2 = __shfl_sync(0xffffffffu, b_own, (e + 2) & 31);
     const float w3 = __shfl_sync(0xffffffffu, b_own, (e + 3) & 31);
-    float v0, v1, v2, v3;
-    if (LEVEL) {
-      v0 = ld_level_f(v + c.x, pol); v1 = ld_level_f(v + c.y, pol);
-      v2 = ld_level_f(v + c.z, pol); v3 = ld_level_f(v + c.w, pol);
-    } else {
-      v0 = ld_keep_f(v + c.x, pol); v1 = ld_keep_f(v + c.y, pol);
-      v2 = ld_keep_f(v + c.z, pol); v3 = ld_keep_f(v + c.w, pol);
-    }
+    const float v0 = ld_keep_f(v + c.x, pol), v1 = ld_keep_f(v + c.y, pol);
+    const float v2 = ld_keep_f(v + c.z, pol), v3 = ld_keep_f(v + c.w, pol);
     acc0 = fmaf(w0, v0, acc0);
     acc1 = fmaf(w1, v1, acc1);
     acc0 = fmaf(w2, v2, acc0);
