@@ -14,8 +14,9 @@ namespace ggp {
 namespace {
 
 // Rows whose FP32 factor needs the FP64 rescue (rescue.cuh) are listed here
-// and recomputed afterwards by factor_rescue_kernel, one thread per row, so
-// that a warp does not stall on the FP64 row of one of its points.  A row
+// and recomputed afterwards (k <= 32: factor_rescue_group_kernel, several rows
+// per warp; above: factor_rescue_kernel, one thread per row), so that a warp
+// does not stall on the FP64 row of one of its points.  A row
 // that finds the list full is recomputed in place.
 struct RescueList {
   int64_t* rows;

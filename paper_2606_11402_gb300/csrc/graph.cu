@@ -1,6 +1,6 @@
 // Graph construction entry points (Sec. 2.2 "Batch construction", Sec. 2.3
-// last paragraph): canonicalised input, k-d tree, preceding kNN, depth by the
-// parallel fixed point, depth-sorted graph order, relabelled neighbour rows,
+// last paragraph): canonicalised input, k-d tree, preceding kNN, depths in one
+// pass over the tree order, depth-sorted graph order, relabelled neighbour rows,
 // and the level tables of the sweeps.  Also import / export / save /
 // load / info / destroy of graph handles.
 #include <algorithm>

@@ -15,8 +15,8 @@
 // covariance value was computed on both sides of the diagonal and a step of
 // the Cholesky used half its lanes on average.  Measured (2^20 uniform points,
 // k = 32, squared exponential, one warp -> eight lanes per point, each call
-// with its dense block): factor 8.9 -> 3.4 ms, NLL gradient 14.6 -> 7.3 ms;
-// factor + NLL + gradient 27.6 -> 11.5 ms.
+// with its dense block): factor 8.9 -> 3.4 ms; factor + NLL + gradient 27.6 ->
+// 12.1 ms.
 #pragma once
 
 #include "pointpair.cuh"
@@ -428,10 +428,9 @@ __device__ __forceinline__ void oct_rescue(OctFactor<K>& f, bool need, float* Sw
 // dkappa/dtheta, in FP32 in the order of the columns; the rows' sums meet in a
 // fixed tree.  As in pair_row_backward the order is kept because the terms
 // cancel; a lane therefore evaluates the values of its rows on both sides of
-// the diagonal (taking each pair once: 2 ms less of 13.1 for factor + NLL +
-// gradient at 2^20, k = 32, but up to 1e-5 of the gradient apart).  Every lane
-// of the warp must call this; `act` says whether the point counts.  The vectors
-// of S are overwritten.
+// the diagonal (taking each pair once saved 2 ms of the 12.1 above and was up
+// to 1e-5 of the gradient apart).  Every lane of the warp must call this; `act`
+// says whether the point counts.  The vectors of S are overwritten.
 template <int K, int KT>
 __device__ __forceinline__ void oct_row_backward(const OctFactor<K>& f, float* S, int r, int k,
                                                  const KernF& kf, float4 xq,

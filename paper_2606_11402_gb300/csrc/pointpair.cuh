@@ -2,9 +2,9 @@
 //
 // The arithmetic is that of pointfactor.cuh (increment or covariance form,
 // left-looking Cholesky with two accumulators, forward solve riding along,
-// compensated sigma^2, backward sweep), element by element and in the same
-// order, so the results equal the group form's bit for bit.  Lane r of a
-// point's pair owns the rows a = 2 s + r (slot s) of M, as packed pairs of
+// compensated sigma^2, backward sweep), element by element and in the order
+// given there.  (In the covariance form the registers hold -kappa, so a value
+// that underflows is a zero of the other sign.)  Lane r of a point's pair owns the rows a = 2 s + r (slot s) of M, as packed pairs of
 // columns in registers; row j of L goes to shared memory when it is complete
 // and both lanes read it back for step j and for the backward sweep.
 //
@@ -25,8 +25,8 @@
 //    warps to choose from.
 // Measured (K = 16, Matern-3/2, unit-Gaussian points): the factor of 2^20 rows
 // takes 13,000 -> 8,100 warp instructions per 32 rows; 2^24 rows, with the
-// dense block and the export, 16.2 -> 10.1 ms; one fit step (value and
-// gradient in one pass) at 2^22 7.9 -> 5.4 ms.  A packed operation takes two
+// dense block and the export, 16.2 -> 9.4 ms; one fit step (value and
+// gradient in one pass) at 2^22 7.9 -> 4.9 ms.  A packed operation takes two
 // issue cycles on this part, so the packing itself saves decoding and code
 // size, not issue slots.
 #pragma once

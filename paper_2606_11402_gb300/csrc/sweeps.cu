@@ -14,7 +14,8 @@
 // synchronises with __syncthreads, since a grid barrier per level costs
 // more than the level's work there: the first run with its field in shared
 // memory, the last with gathers from L2.  Clouds of at most kFlowEntries row
-// entries have no barrier after the first run: a gathered value is its own flag.
+// entries (and kFlowLevel a level) have no barrier after the first run: a gathered
+// value is its own flag.
 //
 // whiten: xi_i = (v_i - b_i . v_c(i)) / sigma_i has no dependencies.  Blocks
 // walk spatial tiles through every level (plus xi_0 = L0^-1 v_0 for the
