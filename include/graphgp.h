@@ -175,8 +175,9 @@ void graphgp_graph_destroy(graphgp_graph_t g);
  * from the stored FP32 sigma.  Pivots below 1e-7 (kappa(0) + nugget) are
  * clamped to that value and counted (see graphgp_sync_status).  The blocks
  * that share the dense block wait for each other; a wait that gave up is
- * reported by graphgp_sync_status.  Allocates stream-ordered scratch (a list of rows for the FP64 pass, FP64 work arrays
- * of 2 n0^2 doubles). */
+ * reported by graphgp_sync_status.  Allocates stream-ordered scratch (a list
+ * of rows for the FP64 pass, work arrays of the dense block of about 20 n0^2
+ * bytes). */
 int graphgp_factor(graphgp_graph_t g, const graphgp_kernel* kern, void* stream,
                    graphgp_factor_t* out);
 
